@@ -16,7 +16,8 @@
  *     (except for sph_step_host, which takes HOST pointers).  The library never
  *     frees caller memory.  Arrays are structure-of-arrays, length n, contiguous.
  *   - The library owns its scratch (cell arrays, sort buffers, packed FP32
- *     copies); it allocates it in sph_init / on first use and frees it in
+ *     copies, neighbour lists: about 700 B per particle, less where the device has
+ *     no room); it allocates it in sph_init / on first use and frees it in
  *     sph_destroy.
  *   - Every call enqueues its work on the stream given to sph_init and returns
  *     after the last launch, EXCEPT where a call documents a host read (the
@@ -137,12 +138,11 @@ typedef struct {
     float alpha_visc;    /* artificial-viscosity strength alpha                      */
     float cfl;           /* dt = cfl * min_i h_i / vsig_i                            */
     float cell_factor;   /* cell side >= cell_factor * max h  (>= 1)                  */
-    int32_t max_h_iter;  /* cap on density passes after the last re-binning          */
+    int32_t max_h_iter;  /* cap on a target's evaluations after the last re-binning  */
     int32_t use_balsara; /* 1: viscosity scaled by the Balsara switch                */
     int32_t kernel;      /* 0: cubic spline (the only kernel)                        */
     uint32_t flags;      /* SPH_FLAG_*                                               */
-    int32_t tile_width;  /* targets per warp work item: 16 (two cells per warp) or   */
-                         /* 32 (one cell per warp); 0 = default (16)                 */
+    int32_t tile_width;  /* targets per warp work item: 16 or 32; 0 = default (32)   */
     int32_t n_boxes;     /* independent periodic boxes batched in one set (0 or 1:   */
                          /* a single box); every box has side box_size               */
     const int64_t *box_offsets; /* HOST, n_boxes + 1 entries, 0 = first <= ... <= */
@@ -276,13 +276,14 @@ int sph_build_cells(sph_ctx *ctx, sph_particles *parts);
  * root that the evaluations so far give is replaced by the bracket's geometric
  * middle) re-running only unconverged particles, until all satisfy
  * |N_w/N_ngb - 1| <= h_tol -- or their bracket is narrower than 2^-21 h, the
- * resolution of the FP32 sums -- or max_h_iter passes ran since the last
- * re-binning.  Rebuilds the cells (permuting the arrays again, restarting the
+ * resolution of the FP32 sums -- or max_h_iter evaluations ran since the last
+ * re-binning.  A pass searches each target's neighbours once, a little beyond h, into a
+ * list and iterates on it; only targets whose h leaves that radius need another pass.  Rebuilds the cells (permuting the arrays again, restarting the
  * iteration) if some h outgrows its cell, at most 8 times per call
  * (SPH_ERR_NOT_CONVERGED beyond that).
  * Writes h, rho, P, c, f, divv, curl, n_ngb.  *iters_out (may be NULL) = passes
  * run.  Requires sph_build_cells on the current positions.  Host read: the
- * unconverged count after each pass.  On the uniform grid, SPH_ERR_PRECISION if a
+ * count of targets left after each pass.  On the uniform grid, SPH_ERR_PRECISION if a
  * converged h is below cell side / SPH_FRAME_RATIO (results are written, and the
  * state counts as having densities, so that sph_force may follow). */
 int sph_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out);

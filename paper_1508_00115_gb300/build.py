@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsph.so")
-SOURCES = ["sph_api.cu", "sph_cells.cu", "sph_pairs.cu", "sph_integrate.cu", "sph_tree.cu", "sph_hpredict.cu",
+SOURCES = ["sph_api.cu", "sph_cells.cu", "sph_pairs.cu", "sph_lists.cu", "sph_integrate.cu", "sph_tree.cu", "sph_hpredict.cu",
            "sph_gravity.cu", "sph_probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-O2", "--extended-lambda",
@@ -33,7 +33,7 @@ def nvcc() -> str:
 
 # the pair kernels (k_density, k_force and their launches) and the cell and tree builds
 # that lay out their work (cell order, leaves, the tiles' targets)
-PAIR_SOURCES = ["sph_pairs.cu", "sph_internal.cuh", "sph_cells.cu", "sph_tree.cu"]
+PAIR_SOURCES = ["sph_pairs.cu", "sph_pairs.cuh", "sph_lists.cu", "sph_internal.cuh", "sph_cells.cu", "sph_tree.cu"]
 
 
 def _digest(files=None) -> str:

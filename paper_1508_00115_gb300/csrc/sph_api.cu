@@ -190,6 +190,39 @@ static int read_counters(sph_ctx *ctx)
     return SPH_OK;
 }
 
+// the largest h that reaches each cell (leaf), which the searches prune with
+static int reach_pass(sph_ctx *ctx, sph_particles *parts)
+{
+    return ctx->adaptive ? tree_leaf_hcur(ctx, parts) : cell_reach(ctx);
+}
+
+// one evaluation of every target at its h, then the force sums: what a step's passes
+// cost (the autotuner's probes)
+static int probe_density(sph_ctx *ctx, sph_particles *parts)
+{
+    if (!lists_apply(ctx)) return run_density_pass(ctx, parts, true, false);
+    ctx->lists.grow = kListGrow;
+    int rc = lists_begin(ctx, false);
+    if (rc == SPH_OK) rc = reach_pass(ctx, parts);
+    if (rc == SPH_OK) rc = run_search(ctx, parts, 0);
+    if (rc == SPH_OK) rc = run_density_lists(ctx, parts, 0, 1, true);
+    if (rc == SPH_OK) rc = run_density_pass(ctx, parts, true, false, true);
+    return rc;
+}
+static int probe_force(sph_ctx *ctx, sph_particles *parts)
+{
+    if (!lists_apply(ctx) || ctx->sym_force) {
+        const int rc = reach_pass(ctx, parts);
+        return rc ? rc : run_force_pass(ctx, parts);
+    }
+    int rc = lists_begin(ctx, true);
+    if (rc == SPH_OK) rc = reach_pass(ctx, parts);
+    if (rc == SPH_OK) rc = run_search(ctx, parts, -1);
+    if (rc == SPH_OK) rc = run_force_lists(ctx, parts);
+    if (rc == SPH_OK) rc = run_force_pass(ctx, parts, false, true);
+    return rc;
+}
+
 // Autotuner: for each candidate schedule, on the current particles, the cell build
 // and one density pass (no h update) followed by one force pass are timed; the
 // density + force pair runs twice and the faster repetition counts, so that one
@@ -231,9 +264,8 @@ static int autotune(sph_ctx *ctx, sph_particles *parts)
             SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_PREC, 0, sizeof(unsigned long long), ctx->stream));
             for (int r = 0; r < 2 && rc == SPH_OK; ++r) {
                 SPH_CUDA(ctx, cudaMemsetAsync(ctx->active, 1, ctx->n, ctx->stream));
-                rc = run_density_pass(ctx, parts, true, false);
-                if (rc == SPH_OK) rc = ctx->adaptive ? tree_leaf_hcur(ctx, parts) : cell_reach(ctx);
-                if (rc == SPH_OK) rc = run_force_pass(ctx, parts);
+                rc = probe_density(ctx, parts);
+                if (rc == SPH_OK) rc = probe_force(ctx, parts);
                 if (rc == SPH_OK) SPH_CUDA(ctx, cudaEventRecord(ev[2 + r], ctx->stream));
             }
             if (rc) break;
@@ -278,9 +310,8 @@ static int autotune(sph_ctx *ctx, sph_particles *parts)
                 rc = build_cells(ctx, parts);
                 if (rc) break;
                 SPH_CUDA(ctx, cudaMemsetAsync(ctx->active, 1, ctx->n, ctx->stream));
-                rc = run_density_pass(ctx, parts, true, false);
-                if (rc == SPH_OK) rc = cell_reach(ctx);
-                if (rc == SPH_OK) rc = run_force_pass(ctx, parts);
+                rc = probe_density(ctx, parts);
+                if (rc == SPH_OK) rc = probe_force(ctx, parts);
                 if (rc) break;
                 SPH_CUDA(ctx, cudaEventRecord(ev[1], ctx->stream));
                 SPH_CUDA(ctx, cudaEventSynchronize(ev[1]));
@@ -299,14 +330,13 @@ static int autotune(sph_ctx *ctx, sph_particles *parts)
         // each timed twice at these smoothing lengths, the faster repetition counting
         ctx->p.flags &= ~SPH_FLAG_TIMING;
         SPH_CUDA(ctx, cudaMemsetAsync(ctx->active, 1, ctx->n, ctx->stream));
-        rc = run_density_pass(ctx, parts, true, false);
-        if (rc == SPH_OK) rc = cell_reach(ctx);
+        rc = probe_density(ctx, parts);
         float t[2] = {1e30f, 1e30f};
         for (int v = 0; v < 2 && rc == SPH_OK; ++v) {
             ctx->sym_force = v == 1;
             for (int r = 0; r < 2 && rc == SPH_OK; ++r) {
                 SPH_CUDA(ctx, cudaEventRecord(ev[0], ctx->stream));
-                rc = run_force_pass(ctx, parts);
+                rc = probe_force(ctx, parts);
                 SPH_CUDA(ctx, cudaEventRecord(ev[1], ctx->stream));
                 SPH_CUDA(ctx, cudaEventSynchronize(ev[1]));
                 float ms = 0.f;
@@ -350,8 +380,8 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
 {
     if (!ctx->built) return fail(ctx, SPH_ERR_STATE, "sph_density needs sph_build_cells on the current positions");
     int n = (int)ctx->n;
-    int iters = 0;
-    int since = 0;     // passes since the last re-binning (each restarts the iteration)
+    int iters = 0;     // passes
+    int since = 0;     // evaluations since the last re-binning (each restarts the iteration)
     int rebinned = 0;  // re-binnings in this call
     unsigned long long unconv = 0;
     if (n > 0 && (ctx->p.flags & SPH_FLAG_AUTOTUNE) && !ctx->tuned) {
@@ -370,31 +400,92 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
         if (rc) return rc;
         rc = reset_h_brackets(ctx);
         if (rc) return rc;
-        bool all_tiles = true;  // first pass (and after a rebuild): every tile
-        if (ctx->bin_mode) {    // individual time-steps: only tiles with a target whose step ends
-            rc = compact_bin_targets(ctx);
-            if (rc) return rc;
-            all_tiles = false;
-        }
+        // passes without lists: every tile at first (and after a rebuild), then those with a
+        // target left; individual time-steps: those with a target whose step ends
+        bool all_tiles = !ctx->bin_mode, compact = ctx->bin_mode;
         SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_PREC, 0, sizeof(unsigned long long), ctx->stream));
-        for (;;) {
-            const bool last = since == ctx->p.max_h_iter - 1;
-            SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_UNCONV, 0, 2 * sizeof(unsigned long long),
-                                          ctx->stream));
-            rc = run_density_pass(ctx, parts, last, !all_tiles);
+        if (lists_apply(ctx)) {
+            rc = ensure_lists(ctx, 0);
             if (rc) return rc;
-            ++iters;
-            ++since;
+        }
+        ctx->lists.ready = false;
+        // adaptive cells take any guess of h, and one off by decades asks for lists of 100,000
+        // names, walked by every Newton step: until a call has converged, passes without lists
+        const bool settled = ctx->lists.settled || !ctx->adaptive;
+        ctx->lists.settled = false;
+        bool use_lists = lists_apply(ctx) && settled;
+        bool fresh = true;     // the next search is the first of the current cells
+        bool partial = false;  // some targets' lists are not in the pool
+        ctx->lists.grow = kListGrow;
+        int pass = 0;          // since lists_begin
+        unsigned long long lost = 0, lost0 = 0;
+        for (;;) {
+            bool last = false;
+            if (use_lists) {
+                if (fresh || pass == kListPasses) {
+                    // (another set of passes keeps the lists at hand out of the force pass)
+                    partial |= !fresh;
+                    lost0 = fresh ? 0 : lost;
+                    rc = lists_begin(ctx, false);
+                    if (rc) return rc;
+                    rc = reach_pass(ctx, parts);
+                    if (rc) return rc;
+                    fresh = false;
+                    pass = 0;
+                }
+                rc = run_search(ctx, parts, pass);
+                if (rc) return rc;
+                rc = run_density_lists(ctx, parts, pass, ctx->p.max_h_iter - since, false);
+                ++pass;
+            } else {
+                if (compact) {
+                    rc = compact_bin_targets(ctx);
+                    if (rc) return rc;
+                    all_tiles = false;
+                }
+                SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_UNCONV, 0, 2 * sizeof(unsigned long long),
+                                              ctx->stream));
+                last = since == ctx->p.max_h_iter - 1;
+                rc = run_density_pass(ctx, parts, last, !all_tiles);
+                compact = true;
+            }
+            if (rc) return rc;
             if (ctx->adaptive && !last) {
                 rc = tree_shrink_count(ctx, parts);
                 if (rc) return rc;
             }
             rc = read_counters(ctx);
             if (rc) return rc;
-            unconv = ctx->h_counters[C_UNCONV];
+            if (use_lists) {
+                if (ctx->h_counters[C_STALE] & 1ull) {
+                    // no page left (the sums did not run): a larger pool, or, where the lists
+                    // would be far too long, passes without them
+                    const int64_t most = std::min<int64_t>(16 * std::max<int64_t>(ctx->cap, 64), kMaxPages);
+                    const int64_t had = ctx->lists.cap_pages;
+                    if ((ctx->h_counters[C_STALE] & 4ull) || had >= most) {
+                        use_lists = false;
+                    } else {
+                        partial |= pass > 1;
+                        rc = ensure_lists(ctx, std::min(most, 2 * had));
+                        if (rc) return rc;
+                        use_lists = lists_apply(ctx);
+                        fresh = true;
+                    }
+                    continue;
+                }
+                lost = lost0 + ctx->h_counters[C_LOST];
+                since += (int)ctx->h_counters[C_PASS + 4 * (pass - 1) + 3];
+                unconv = ctx->h_counters[C_PASS + 4 * (pass - 1)];
+            } else {
+                ++since;
+                unconv = ctx->h_counters[C_UNCONV];
+            }
+            ++iters;
             if (unconv == 0 || last) break;
-            // adaptive: lists much longer than the current h need (1 leaf in 16)
-            const bool shrunk = ctx->adaptive && ctx->h_counters[C_SHRINK] * 16 > (unsigned long long)ctx->tree.n_leaves;
+            // adaptive: lists much longer than the current h need (1 leaf in 16); the sums over
+            // neighbour lists iterate to the end, so that few are left to gain from new cells
+            const bool few_left = use_lists && unconv * 8 < (unsigned long long)n;
+            const bool shrunk = ctx->adaptive && !few_left && ctx->h_counters[C_SHRINK] * 16 > (unsigned long long)ctx->tree.n_leaves;
             const bool outgrown = ctx->h_counters[C_HFLAG] != 0;
             if (outgrown && rebinned >= kMaxRebins) {
                 char buf[160];
@@ -411,25 +502,33 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
                 ctx->st.rebuilds++;
                 ++rebinned;
                 since = 0;
+                use_lists = lists_apply(ctx) && settled;
+                fresh = true;
+                partial = false;
                 rc = init_active(ctx);
                 if (rc) return rc;
                 rc = reset_h_brackets(ctx);  // slots were permuted
                 if (rc) return rc;
                 SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_PREC, 0, sizeof(unsigned long long), ctx->stream));
-                all_tiles = true;
-                if (ctx->bin_mode) {
-                    rc = compact_bin_targets(ctx);
-                    if (rc) return rc;
-                    all_tiles = false;
-                }
-            } else {
-                rc = ctx->adaptive ? compact_active_leaf_tiles(ctx) : compact_active_tiles(ctx);
-                if (rc) return rc;
-                all_tiles = false;
+                all_tiles = !ctx->bin_mode;
+                compact = ctx->bin_mode;
             }
+        }
+        unconv += lost;
+        if (use_lists && !partial && ctx->h_counters[C_GROWN]) {
+            rc = run_mark(ctx, parts);
+            if (rc) return rc;
         }
         rc = sync_h(ctx, parts);
         if (rc) return rc;
+        if (lists_apply(ctx)) {
+            // the force pass searches again where the lists at hand are not all there
+            if (!use_lists || partial)
+                SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_STALE, 2, 1, ctx->stream));
+            ctx->lists.ready = true;
+            ctx->lists.settled = unconv == 0;
+            ctx->lists.stale = !use_lists || partial || (ctx->h_counters[C_STALE] & 3ull) != 0 || ctx->h_counters[C_GROWN] != 0;
+        }
     }
     if (iters_out) *iters_out = iters;
     ctx->density_valid = true;
@@ -453,17 +552,32 @@ static int do_force(sph_ctx *ctx, sph_particles *parts)
 {
     if (!ctx->density_valid) return fail(ctx, SPH_ERR_STATE, "sph_force needs sph_density on the current state");
     if (ctx->n > 0) {
+        const bool lists = ctx->lists.ready && lists_apply(ctx) && !ctx->sym_force;
+        int rc = SPH_OK;
         // uniform grid: reach of every cell for r < max(h_i, h_j) (adaptive cells
         // prune every source with its own h)
-        int rc = ctx->adaptive ? tree_leaf_hcur(ctx, parts) : cell_reach(ctx);
+        if (!lists || ctx->lists.stale) rc = reach_pass(ctx, parts);
         if (rc) return rc;
-        if (ctx->bin_mode) {  // individual time-steps: the tiles of the targets whose step ends
+        if (ctx->bin_mode && (!lists || ctx->lists.stale)) {
+            // individual time-steps: the tiles of the targets whose step ends
             rc = init_active(ctx);
             if (rc) return rc;
             rc = compact_bin_targets(ctx);
             if (rc) return rc;
         }
-        rc = run_force_pass(ctx, parts, ctx->bin_mode);
+        if (lists) {
+            rc = lists_begin(ctx, true);
+            if (rc) return rc;
+            if (ctx->lists.stale) {
+                rc = run_search(ctx, parts, -1);
+                if (rc) return rc;
+            }
+            rc = run_force_lists(ctx, parts);
+            if (rc) return rc;
+            if (ctx->lists.stale) rc = run_force_pass(ctx, parts, ctx->bin_mode, true);
+        } else {
+            rc = run_force_pass(ctx, parts, ctx->bin_mode);
+        }
         if (rc) return rc;
     }
     ctx->hydro_valid = true;
@@ -477,6 +591,7 @@ static int do_build(sph_ctx *ctx, sph_particles *parts)
     int rc = build_cells(ctx, parts);
     timer_end(ctx, end);
     ctx->hydro_valid = false;
+    ctx->lists.ready = false;
     return rc;
 }
 
@@ -543,6 +658,8 @@ static int hydro(sph_ctx *ctx, sph_particles *parts, bool in_step = false)
     const bool collect = in_step && ctx->hp.col_feats;
     if (predict) {
         rc = hp_apply_step(ctx, parts);
+        if (rc) return rc;
+        rc = sync_h(ctx, parts);  // the searches take the sources' reach from there
         if (rc) return rc;
     } else if (collect) {
         rc = hp_features(ctx, parts);
@@ -750,7 +867,7 @@ static int do_step_bins(sph_ctx *ctx, sph_particles *parts, double dt_max, int l
 __global__ void k_step_flags(unsigned long long *c)
 {
     unsigned long long f = 0;
-    if (c[C_UNCONV]) f |= 1ull;
+    if (c[C_UNCONV] || c[C_LOST]) f |= 1ull;
     if (c[C_HFLAG]) f |= 2ull;
     if (c[C_PREC]) f |= 4ull;
     if (c[C_TCERR]) f |= 8ull;
@@ -772,6 +889,8 @@ static int graph_step(sph_ctx *ctx, sph_particles *parts, double dt, int passes)
     if (ctx->p.flags & SPH_FLAG_HPREDICT) {
         rc = hp_apply_step(ctx, parts);
         if (rc) return rc;
+        rc = sync_h(ctx, parts);
+        if (rc) return rc;
     }
     const int n = (int)ctx->n;
     SPH_CUDA(ctx, cudaMemsetAsync(ctx->active, 1, n, ctx->stream));
@@ -779,22 +898,51 @@ static int graph_step(sph_ctx *ctx, sph_particles *parts, double dt, int passes)
     if (rc) return rc;
     SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_UNCONV, 0, 2 * sizeof(unsigned long long), ctx->stream));
     SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_PREC, 0, sizeof(unsigned long long), ctx->stream));
+    const bool lists = lists_apply(ctx);
+    ctx->lists.grow = kListGrow;
+    SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_LOST, 0, sizeof(unsigned long long), ctx->stream));
+    if (lists) {
+        rc = lists_begin(ctx, false);
+        if (rc) return rc;
+        rc = reach_pass(ctx, parts);
+        if (rc) return rc;
+    }
     for (int p = 0; p < passes; ++p) {
-        if (p > 0) {
+        const bool last = p == passes - 1;
+        if (lists) {
+            // the passes after the first run where the one before left targets; the kernel
+            // without lists, over every tile, only where the lists had no room
+            rc = run_search(ctx, parts, p);
+            if (rc) return rc;
+            rc = run_density_lists(ctx, parts, p, ctx->p.max_h_iter, last);
+            if (rc) return rc;
+        } else if (p > 0) {
             rc = ctx->adaptive ? compact_active_leaf_tiles(ctx) : compact_active_tiles(ctx);
             if (rc) return rc;
-            SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_UNCONV, 0, sizeof(unsigned long long), ctx->stream));
         }
-        rc = run_density_pass(ctx, parts, p == passes - 1, p > 0);
+        if (p > 0) SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_UNCONV, 0, sizeof(unsigned long long), ctx->stream));
+        rc = run_density_pass(ctx, parts, last, p > 0 && !lists, lists);
         if (rc) return rc;
     }
     k_step_flags<<<1, 1, 0, ctx->stream>>>(ctx->counters);
     SPH_LAUNCH(ctx, "step flags");
+    if (lists) {
+        rc = run_mark(ctx, parts);
+        if (rc) return rc;
+    }
     rc = sync_h(ctx, parts);
     if (rc) return rc;
-    rc = ctx->adaptive ? tree_leaf_hcur(ctx, parts) : cell_reach(ctx);  // adaptive: sources' h per leaf
+    rc = reach_pass(ctx, parts);
     if (rc) return rc;
-    rc = run_force_pass(ctx, parts);
+    if (lists && !ctx->sym_force) {
+        rc = lists_begin(ctx, true);
+        if (rc) return rc;
+        rc = run_search(ctx, parts, -1);
+        if (rc) return rc;
+        rc = run_force_lists(ctx, parts);
+        if (rc) return rc;
+    }
+    rc = run_force_pass(ctx, parts, false, lists && !ctx->sym_force);
     if (rc) return rc;
     ctx->predict = false;
     rc = kick(ctx, parts);
@@ -853,6 +1001,14 @@ static int do_steps(sph_ctx *ctx, sph_particles *parts, int n_steps, double dt, 
         rc = tree_prepare_device(ctx, &tree_sig);
         if (rc) return rc;
     }
+    if (lists_apply(ctx)) {  // the pages the last searches took, and half as many again at least
+        rc = read_counters(ctx);
+        if (rc) return rc;
+        const int64_t used = (int64_t)ctx->h_counters[C_PAGES];
+        if (used + used / 2 > ctx->lists.cap_pages) ctx->lists.ready = false;
+        rc = ensure_lists(ctx, used + used / 2 > ctx->lists.cap_pages ? 2 * used : 0);
+        if (rc) return rc;
+    }
     // capture one step on a private stream (the caller's may be the legacy default
     // stream, which cannot be captured); the graph is then launched on the caller's
     // stream.  The timing flag is suspended while capturing.  A graph captured for
@@ -862,7 +1018,7 @@ static int do_steps(sph_ctx *ctx, sph_particles *parts, int n_steps, double dt, 
         if (rc) return rc;
     }
     sph_ctx::GraphKey key{*parts, dt > 0 ? dt : 0.0, ctx->n, ctx->grid.n_cells, ctx->grid.key_bits, passes, ctx->tile_w,
-                          tree_sig, ctx->sym_force};
+                          tree_sig, ctx->sym_force, ctx->lists.pages, ctx->lists.cap_pages};
     if (!ctx->step_exec || !(key == ctx->graph_key)) {
         if (!ctx->cap_stream) SPH_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
         const uint32_t flags = ctx->p.flags;
@@ -927,6 +1083,7 @@ static int do_steps(sph_ctx *ctx, sph_particles *parts, int n_steps, double dt, 
     ctx->hydro_valid = true;
     ctx->density_valid = true;
     ctx->built = true;
+    ctx->lists.ready = false;
     sph_conserved tmp;
     rc = conserved_read(ctx, out ? out : &tmp);
     if (rc) return rc;
@@ -988,7 +1145,7 @@ int sph_init(sph_ctx **out, const sph_params *p, int device, void *cuda_stream)
     c->device = device;
     c->stream = (cudaStream_t)cuda_stream;
     c->n = p->n;
-    c->tile_w = p->tile_width == 32 ? 32 : 16;
+    c->tile_w = p->tile_width == 16 ? 16 : 32;
     c->adaptive = (p->flags & SPH_FLAG_ADAPTIVE) != 0;
     c->sym_force = (p->flags & SPH_FLAG_SYMMETRIC) != 0 && !c->adaptive;
     c->leaf_max = p->leaf_max > 0 ? p->leaf_max : 64;
@@ -1370,6 +1527,7 @@ void sph_destroy(sph_ctx *ctx)
     free_particles(ctx);
     free_bins(ctx);
     free_tree(ctx);
+    free_lists(ctx);
     cudaFree(ctx->axis);
     hp_free(ctx);
     cudaFree(ctx->cell_start);

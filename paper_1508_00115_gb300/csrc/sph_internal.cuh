@@ -68,8 +68,26 @@ enum Counter {
     C_TMIN = 26,      // individual time-steps: earliest step end
     C_LIMACT = 27,    // time-step limiter: particles in the active list
     C_TCERR = 28,     // learned h: a tensor-core (mbarrier) wait of the inference ran out
-    C_NCOUNTERS = 29
+    C_PAGES = 29,     // neighbour lists: pages handed out
+    C_STALE = 30,     // neighbour lists: bit 0 the pool ran out (or a leaf is too large for the
+                      // names), bit 1 some targets' lists were lost, bit 2 with bit 0: more
+                      // pages would not help
+    C_FOVF = 31,      // neighbour lists: the force pass's own search ran out of pages
+    C_LOST = 32,      // targets that used up their evaluations without converging
+    C_FTICKET = 33,   // list sums of the force pass: tickets of the search and of the sums
+    C_PASS = 35,      // list sums, four per density pass: targets that need another pass, tickets
+                      // of the search and of the sums, most evaluations of a target left
+    C_GROWN = C_PASS + 4 * 8,  // neighbour lists: targets whose h outgrew the radius their
+                               // neighbours searched with
+    C_DIRTY,                   // ... and the targets among those neighbours that miss them
+    C_NCOUNTERS
 };
+// List radius / h.  The h of a step moves by a few per cent at most: 1.04^3 = 12 % more
+// names buy that nearly no particle needs a second search.  (1.12 for a first search from a
+// caller's guess, whose longer lists spare most of a second search, was slower: 25.5 against
+// 22.2 ms on 2 M clustered particles with h 3 % off, 0.77 against 0.60 on 32^3 random ones.)
+constexpr float kListGrow = 1.04f;
+constexpr int kListPasses = 8;  // density passes between two lists_begin
 
 // Cell grid of one periodic box (every box has side box_size; boxes are batched
 // by concatenating their particle ranges and their cell numberings).
@@ -139,11 +157,12 @@ struct AdaptiveTree {
     float *leaf_scale = nullptr; // coordinate scale of the leaf's pair arithmetic (FP32 band width)
     uint32_t *list_off = nullptr; // neighbour-list offsets, n_leaves + 1
     float4 *list = nullptr;     // {offset between leaf centres, neighbour leaf}
+    int *list_slot = nullptr;   // first slot of the entry's leaf
     uint32_t *h_u32 = nullptr;  // pinned scratch for host reads
     int *h_i32 = nullptr;
     int64_t cap_keys = 0, cap_keys2 = 0, cap_leaf_of = 0, cap_tord = 0, cap_act_ord = 0, cap_nact_leaf = 0, cap_node_at = 0, cap_top = 0, cap_nodes = 0,
             cap_front = 0, cap_front2 = 0, cap_bounds = 0, cap_nkids = 0, cap_node_leaf = 0, cap_leaf_node = 0,
-            cap_leaf_rng = 0, cap_leaf_cen = 0, cap_leaf_h = 0, cap_leaf_scale = 0, cap_list_off = 0, cap_list = 0,
+            cap_leaf_rng = 0, cap_leaf_cen = 0, cap_leaf_h = 0, cap_leaf_scale = 0, cap_list_off = 0, cap_list = 0, cap_list_slot = 0,
             cap_leaf_lo = 0, cap_leaf_hi = 0;
     int n_nodes = 0, n_leaves = 0;
     int64_t n_entries = 0;
@@ -171,6 +190,23 @@ struct HPredictor {
     // sample collection during sph_step (caller's device buffers)
     float *col_feats = nullptr, *col_target = nullptr;
     int64_t col_cap = 0, col_n = 0;
+};
+
+constexpr int64_t kMaxPages = (int64_t)1 << 27;  // pages of the neighbour lists: 2^32 names
+// neighbour lists of the pair sums (sph_lists.cu)
+struct ListPool {
+    uint32_t *pages = nullptr;  // 32 names each
+    int *next = nullptr;        // per chunk of a list: its pages, the next chunk
+    int *head = nullptr, *cnt = nullptr;  // per slot: first page, names
+    float *radius = nullptr;    // per slot: list radius
+    int *rows = nullptr;        // 4 x cap: targets left by the last two passes, grown, dirty
+    uint8_t *mark = nullptr;    // dirty targets (zero between the force passes)
+    int64_t cap = 0, cap_pages = 0;
+    bool off = false;           // no room on the device
+    bool ready = false;         // lists of the current cells, from the last density call
+    bool stale = false;         // ... that do not serve the force pass
+    bool settled = false;       // the last density call converged
+    float grow = 1.f;           // list radius / h of the last density call
 };
 
 struct Grid {
@@ -279,11 +315,13 @@ struct sph_ctx {
         int key_bits, passes, tile_w;
         uint64_t tree_sig;  // adaptive cells: arrays and capacities the captured build uses
         bool sym;           // symmetric force pass
+        const void *list_pages;  // neighbour-list pool
+        int64_t list_cap;
         bool operator==(const GraphKey &o) const
         {
             return memcmp(&parts, &o.parts, sizeof parts) == 0 && dt == o.dt && n == o.n && n_cells == o.n_cells &&
                    key_bits == o.key_bits && passes == o.passes && tile_w == o.tile_w && tree_sig == o.tree_sig &&
-                   sym == o.sym;
+                   sym == o.sym && list_pages == o.list_pages && list_cap == o.list_cap;
         }
     } graph_key{};
     int64_t graph_launches = 0;  // kernels in one captured step
@@ -325,6 +363,8 @@ struct sph_ctx {
     float4 *sym_slot = nullptr;
     unsigned *sym_vsig = nullptr;
     int64_t sym_cap = 0;
+
+    sph::ListPool lists;  // neighbour lists
 
     // statistics
     sph_stats st{};
@@ -398,11 +438,23 @@ int hp_train(sph_ctx *ctx, const float *X, const float *Y, int64_t n, int epochs
 void hp_free(sph_ctx *ctx);
 void free_tree(sph_ctx *ctx);                                   // sph_tree.cu
 int cell_keys_out(sph_ctx *ctx, int32_t *dev_keys);             // sph_cells.cu
-int run_density_pass(sph_ctx *ctx, sph_particles *parts, bool last_pass, bool active_list);  // sph_pairs.cu
+// (if_no_lists: the kernel runs only where the lists could not be used)
+int run_density_pass(sph_ctx *ctx, sph_particles *parts, bool last_pass, bool active_list,
+                     bool if_no_lists = false);                            // sph_pairs.cu
+// sums over neighbour lists, sph_lists.cu
+bool lists_apply(const sph_ctx *ctx);
+int ensure_lists(sph_ctx *ctx, int64_t pages);  // (outside captures)
+void free_lists(sph_ctx *ctx);
+int lists_begin(sph_ctx *ctx, bool force);
+int run_search(sph_ctx *ctx, sph_particles *parts, int pass);
+int run_density_lists(sph_ctx *ctx, sph_particles *parts, int pass, int budget, bool last_pass);
+int run_mark(sph_ctx *ctx, sph_particles *parts);
+int run_force_lists(sph_ctx *ctx, sph_particles *parts);
 int compact_active_tiles(sph_ctx *ctx);                                    // sph_pairs.cu
 int compact_active_leaf_tiles(sph_ctx *ctx);  // adaptive cells: tiles of active targets only  // sph_tree.cu
 int order_tiles(sph_ctx *ctx, int4 *tiles, const int *n_tiles);  // adaptive: longest-first tile groups  // sph_tree.cu
-int run_force_pass(sph_ctx *ctx, sph_particles *parts, bool active_list = false);  // sph_pairs.cu
+int run_force_pass(sph_ctx *ctx, sph_particles *parts, bool active_list = false,
+                   bool if_no_lists = false);  // sph_pairs.cu
 int run_gravity_pass(sph_ctx *ctx, double G, double eps, float *ax, float *ay, float *az, float *phi);  // sph_gravity.cu
 int ensure_sym(sph_ctx *ctx);  // slot arrays of the symmetric force pass           // sph_pairs.cu
 int sync_h(sph_ctx *ctx, sph_particles *parts);                            // sph_pairs.cu

@@ -26,14 +26,13 @@
 // neighbour sets are exact.
 #include <algorithm>
 
-#include "sph_internal.cuh"
+#include "sph_pairs.cuh"
 
 namespace sph {
 
 constexpr int kBatchD = 128;  // staged survivors per tile, density (4 hit-mask words)
 constexpr int kBatchF = 128;  // staged survivors per tile, force
 constexpr int kSlotF = 132;   // floats per staged-coordinate array (>= kBatchD, even: 8-byte aligned pairs)
-constexpr int kPairThreads = 256;
 // Adaptive cells (leaf lists): the tiles' targets span a range of h, so their hit
 // counts in a batch differ widely.  The density and force passes therefore cut a
 // batch's hits into equal contiguous ranges, one per lane (the balanced walk of
@@ -48,45 +47,6 @@ constexpr int kWalkBytes = 148;   // force pass, list mode: the balanced walk's 
 constexpr int kDensityBlocks = 2;  // resident blocks per SM the density kernel is compiled for
 constexpr int kForceBlocks = 2;      // leaf lists (adaptive cells): 3 would spill (328 B at 80 registers)
 constexpr int kForceBlocksU = 3;     // uniform grid: a third block per SM outweighs a few spilled values
-// Padding sources sit at -kFar and target-less lanes at +kFar: the squared distance
-// between either and anything else overflows to +inf, so no test can pass.
-constexpr float kFar = 1e30f;
-// an h bracket end at or above this is open (the bytes 0x7f7f7f7f read 3.39e38)
-constexpr float kHUnbounded = 3e38f;
-// relative width of an h bracket at which the iteration stops refining (2^-21: 4 to 8
-// FP32 ulps of h); near the root the FP32 neighbour sums are noisy at about this level
-// of h, so that for particles whose N_w is very sensitive to h a tolerance far below
-// 1e-5 may have no FP32 h that meets it
-constexpr float kHResolution = 4.76837158e-7f;
-
-// Neighbour cells in visiting order: the own cell, then each of the 13 directions
-// of a half stencil followed by its opposite, so that every staged batch mixes
-// cells on both sides of the tile and the lanes' hit counts stay balanced.
-__constant__ signed char kOrder[27][3] = {
-    {0, 0, 0},   {1, 0, 0},   {-1, 0, 0},  {0, 1, 0},   {0, -1, 0},   {0, 0, 1},  {0, 0, -1},
-    {1, 1, 0},   {-1, -1, 0}, {1, -1, 0},  {-1, 1, 0},  {1, 0, 1},    {-1, 0, -1}, {1, 0, -1},
-    {-1, 0, 1},  {0, 1, 1},   {0, -1, -1}, {0, 1, -1},  {0, -1, 1},   {1, 1, 1},  {-1, -1, -1},
-    {1, 1, -1},  {-1, -1, 1}, {1, -1, 1},  {-1, 1, -1}, {-1, 1, 1},   {1, -1, -1}};
-
-// Radius-2 stencils visit the 27 cells above, in that order, then the 98 cells at
-// distance two (z, y, x lexicographic), so a tile's summation order never depends
-// on which stencil its warp runs.
-__constant__ signed char kOuter[98][3] = {
-    {-2, -2, -2}, {-1, -2, -2}, {0, -2, -2}, {1, -2, -2}, {2, -2, -2}, {-2, -1, -2}, {-1, -1, -2},
-    {0, -1, -2}, {1, -1, -2}, {2, -1, -2}, {-2, 0, -2}, {-1, 0, -2}, {0, 0, -2}, {1, 0, -2},
-    {2, 0, -2}, {-2, 1, -2}, {-1, 1, -2}, {0, 1, -2}, {1, 1, -2}, {2, 1, -2}, {-2, 2, -2},
-    {-1, 2, -2}, {0, 2, -2}, {1, 2, -2}, {2, 2, -2}, {-2, -2, -1}, {-1, -2, -1}, {0, -2, -1},
-    {1, -2, -1}, {2, -2, -1}, {-2, -1, -1}, {2, -1, -1}, {-2, 0, -1}, {2, 0, -1}, {-2, 1, -1},
-    {2, 1, -1}, {-2, 2, -1}, {-1, 2, -1}, {0, 2, -1}, {1, 2, -1}, {2, 2, -1}, {-2, -2, 0},
-    {-1, -2, 0}, {0, -2, 0}, {1, -2, 0}, {2, -2, 0}, {-2, -1, 0}, {2, -1, 0}, {-2, 0, 0},
-    {2, 0, 0}, {-2, 1, 0}, {2, 1, 0}, {-2, 2, 0}, {-1, 2, 0}, {0, 2, 0}, {1, 2, 0},
-    {2, 2, 0}, {-2, -2, 1}, {-1, -2, 1}, {0, -2, 1}, {1, -2, 1}, {2, -2, 1}, {-2, -1, 1},
-    {2, -1, 1}, {-2, 0, 1}, {2, 0, 1}, {-2, 1, 1}, {2, 1, 1}, {-2, 2, 1}, {-1, 2, 1},
-    {0, 2, 1}, {1, 2, 1}, {2, 2, 1}, {-2, -2, 2}, {-1, -2, 2}, {0, -2, 2}, {1, -2, 2},
-    {2, -2, 2}, {-2, -1, 2}, {-1, -1, 2}, {0, -1, 2}, {1, -1, 2}, {2, -1, 2}, {-2, 0, 2},
-    {-1, 0, 2}, {0, 0, 2}, {1, 0, 2}, {2, 0, 2}, {-2, 1, 2}, {-1, 1, 2}, {0, 1, 2},
-    {1, 1, 2}, {2, 1, 2}, {-2, 2, 2}, {-1, 2, 2}, {0, 2, 2}, {1, 2, 2}, {2, 2, 2},};
-
 // SPH_FLAG_AXIS_SWEEP: for stencil cell o (kOrder index) the direction d of the 13
 // half-stencil axes with kOrder[o] = sign * axis d, and |axis d| (1, sqrt 2, sqrt 3)
 __constant__ signed char kOrderAxis[27][2] = {
@@ -111,108 +71,6 @@ __device__ __forceinline__ float sweep_limit(int o, float L, float rlim, float l
     return rlim + tmax - len * L + 1e-5f * L;
 }
 
-// The sources of a tile's leaf list as one stream (adaptive cells).  The TW entries
-// of a window are fetched at once (lane tl: entry wb + tl), their particle counts are
-// prefix-summed across the TW lanes, and chunk ch of the window covers stream
-// positions [ch TW, ch TW + TW): leaves much smaller than TW share a chunk instead of
-// each leaving lanes idle.  The stream order -- entries in list order, particles in
-// slot order -- is that of the entries taken one by one.
-template <int TW>
-struct ListStream {
-    int wb = -TW;  // first entry of the window (warp-uniform)
-    int incl = 0;  // prefix count of the window's entries up to this lane's, inclusive
-    int st = 0;    // stream position of this lane's entry (its first particle)
-    int sb = 0;    // first slot of this lane's entry minus its stream position
-    int tot = 0;   // particles in this tile's window
-    float px = 0.f, py = 0.f, pz = 0.f;  // offset of this lane's entry
-
-    // next window (warp-uniform); false once the longest list of the warp is done;
-    // *nchunk = the warp's largest chunk count of the window.  An entry whose leaf box
-    // (moved by the entry's offset) lies beyond reach of the tile's box contributes no
-    // sources: the staging would reject every one of them.  Reach: sqrt(reach2) for the
-    // density (targets' h); for the force (FORCE) the larger of the targets' h and the
-    // leaf's largest current h (set before the force pass).
-    template <bool FORCE>
-    __device__ __forceinline__ bool next(const float4 *__restrict__ list, const int2 *__restrict__ rng,
-                                         const float4 *__restrict__ blo, const float4 *__restrict__ bhi, uint32_t e0,
-                                         int ne, int ncell, int tl, int &nchunk, float lox, float hix, float loy,
-                                         float hiy, float loz, float hiz, float reach2, float H, float L)
-    {
-        wb += TW;
-        if (wb >= ncell) return false;
-        int c = 0, b = 0;
-        px = py = pz = 0.f;
-        if (wb + tl < ne) {
-            const float4 en = list[e0 + (uint32_t)(wb + tl)];
-            const int lf = __float_as_int(en.w);
-            const int2 r = rng[lf];
-            b = r.x;
-            c = r.y - r.x;
-            px = en.x;
-            py = en.y;
-            pz = en.z;
-            const float4 lo = blo[lf], hi = bhi[lf];
-            const float gx = fmaxf(fmaxf(lo.x + px - hix, lox - (hi.x + px)), 0.f);
-            const float gy = fmaxf(fmaxf(lo.y + py - hiy, loy - (hi.y + py)), 0.f);
-            const float gz = fmaxf(fmaxf(lo.z + pz - hiz, loz - (hi.z + pz)), 0.f);
-            float r2 = reach2;
-            if (FORCE) {
-                const float m = fmaxf(H, lo.w);
-                r2 = m * m * (1.f + kPruneMargin) + 2.f * kBandK * m * (m + L);
-            }
-            if (fmaf(gx, gx, fmaf(gy, gy, gz * gz)) > r2 * 1.00001f) c = 0;
-        }
-        // the window's non-empty entries moved to the front (list order kept), so that
-        // the lookup below meets no empty entry before the last non-empty one
-        {
-            const int g = TW == 32 ? 0 : (int)(threadIdx.x & 31) / TW;
-            const unsigned gm = TW == 32 ? kFull : (((1u << TW) - 1u) << (TW * g));
-            const unsigned mine = __ballot_sync(kFull, c > 0) & gm;
-            const unsigned src = __fns(mine, (unsigned)(TW * g), tl + 1);
-            const bool has = src < 32u;
-            const int sl = has ? (int)src : (int)(threadIdx.x & 31);
-            c = __shfl_sync(kFull, c, sl);
-            b = __shfl_sync(kFull, b, sl);
-            px = __shfl_sync(kFull, px, sl);
-            py = __shfl_sync(kFull, py, sl);
-            pz = __shfl_sync(kFull, pz, sl);
-            if (!has) c = 0;
-        }
-        incl = c;
-#pragma unroll
-        for (int d = 1; d < TW; d <<= 1) {
-            const int v = __shfl_up_sync(kFull, incl, d, TW);
-            if (tl >= d) incl += v;
-        }
-        st = incl - c;
-        sb = b - st;
-        tot = __shfl_sync(kFull, incl, TW - 1, TW);
-        nchunk = (int)__reduce_max_sync(kFull, (unsigned)((tot + TW - 1) / TW));
-        return true;
-    }
-
-    // slot j, validity and entry offset of the stream position base + tl of chunk
-    // base (every lane calls it): the entry holding position base is the number of
-    // entries that end at or before it; each entry that starts inside the chunk, at
-    // or before the lane's position, adds one
-    __device__ __forceinline__ void slot(int base, int tl, int &j, bool &v, float &sx, float &sy,
-                                         float &sz) const
-    {
-        const int g = TW == 32 ? 0 : (int)(threadIdx.x & 31) / TW;  // tile of the lane within the warp
-        const unsigned gm = TW == 32 ? kFull : (((1u << TW) - 1u) << (TW * g));
-        const bool inside = st > base && st < base + TW && st < incl;
-        const unsigned starts = __reduce_or_sync(kFull, inside ? 1u << (TW * g + st - base) : 0u) >> (TW * g);
-        const int eb = __popc(__ballot_sync(kFull, incl <= base) & gm);
-        const int e = min(eb + __popc(starts & ((2u << tl) - 2u)), TW - 1);
-        const int q = base + tl;
-        j = __shfl_sync(kFull, sb, e, TW) + q;
-        sx = __shfl_sync(kFull, px, e, TW);
-        sy = __shfl_sync(kFull, py, e, TW);
-        sz = __shfl_sync(kFull, pz, e, TW);
-        v = q < tot;
-    }
-};
-
 struct DensityArgs {
     const float4 *__restrict__ pos4;
     const float4 *__restrict__ vel4;
@@ -224,6 +82,7 @@ struct DensityArgs {
     const double *__restrict__ z;
     const int64_t *__restrict__ ids;
     const float *__restrict__ upred;
+    const unsigned long long *__restrict__ run_if;  // non-null: run only if bit 0 of it is set
     uint8_t *active;
     float *h;
     float *h_lo, *h_hi;  // bracket of the root of N_w(h) = N_ngb
@@ -249,30 +108,6 @@ struct DensityArgs {
     int use_balsara;
     int last_pass;
 };
-
-// reductions over the TW lanes of a tile (xor offsets < TW stay inside the tile)
-template <int TW>
-__device__ __forceinline__ float tile_min(float v)
-{
-#pragma unroll
-    for (int o = TW / 2; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(kFull, v, o));
-    return v;
-}
-template <int TW>
-__device__ __forceinline__ float tile_max(float v)
-{
-#pragma unroll
-    for (int o = TW / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kFull, v, o));
-    return v;
-}
-__device__ __forceinline__ unsigned long long warp_sum_ull(unsigned long long v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
-}
-
-__device__ __forceinline__ int wrapc(int j, int nc) { return j < 0 ? j + nc : (j >= nc ? j - nc : j); }
 
 // Pop the lowest set bit of a 128-bit mask held in four words; returns its index.
 __device__ __forceinline__ int pop_bit(unsigned &m0, unsigned &m1, unsigned &m2, unsigned &m3)
@@ -310,34 +145,6 @@ __device__ __forceinline__ void drop_hits(uint4 &M, int r)
     M.w = keep_after(M.w, r);
 }
 
-// Cubic spline of support 1 without its normalisation sigma, in truncated-power form:
-// w/sigma = 2(1-q)^3_+ - 8(1/2-q)^3_+,  (dw/dq)/sigma = -6(1-q)^2_+ + 24(1/2-q)^2_+
-// (identical to the piecewise polynomial; branch-free).
-__device__ __forceinline__ void spline_u(float q, float &w, float &dw)
-{
-    const float a = fmaxf(1.f - q, 0.f), b = fmaxf(0.5f - q, 0.f);
-    const float a2 = a * a, b2 = b * b;
-    w = fmaf(-8.f * b2, b, 2.f * a2 * a);
-    dw = fmaf(24.f, b2, -6.f * a2);
-}
-__device__ __forceinline__ float spline_dw_u(float q)
-{
-    const float a = fmaxf(1.f - q, 0.f), b = fmaxf(0.5f - q, 0.f);
-    return fmaf(24.f * b, b, -6.f * a * a);
-}
-
-// Partial force sums of one target: a, du/dt and the largest v_sig.
-struct ForceSum {
-    float x = 0.f, y = 0.f, z = 0.f, u = 0.f, v = 0.f;
-    // store into slot idx (sums into the float4, v_sig beside) and start again
-    __device__ __forceinline__ void put(float4 *s4, float *sv, int idx)
-    {
-        s4[idx] = make_float4(x, y, z, u);
-        sv[idx] = v;
-        x = y = z = u = v = 0.f;
-    }
-};
-
 // Partial density sums of one target: {sum m w, sum w, sum q w', sum m (3 w + q w')}
 // and {sum (v_ij . d) m w'/r, the three components of the curl sum}.
 struct DensSum {
@@ -351,41 +158,12 @@ struct DensSum {
     }
 };
 
-// The pair term of the force pass (Sec. 2: the grad-h pressure force with the
-// Monaghan viscosity and its Balsara switch, and du/dt) of target i (1/h_i, 1/h_i^4,
-// v_i, thermo_i = {rho, f P / rho^2, c, B}) and source j (h_j, {v_j, m_j}, thermo_j)
-// at d = p_i - p_j, r2 = |d|^2 > 0; in_i, in_j: r < h_i, r < h_j.
-__device__ __forceinline__ void force_term(float dx, float dy, float dz, float r2, bool in_i, bool in_j, float hinv,
-                                           float hinv4, const float4 vi, const float4 ti, float hj, const float4 vj,
-                                           const float4 tj, float alpha, ForceSum &f)
-{
-    const float rinv = rsqrtf(r2);
-    const float r = r2 * rinv;
-    const float hjinv = __fdividef(1.f, hj);
-    const float hj2inv = hjinv * hjinv;
-    const float dWi = in_i ? kSigma * spline_dw_u(r * hinv) * hinv4 : 0.f;
-    const float dWj = in_j ? kSigma * spline_dw_u(r * hjinv) * (hj2inv * hj2inv) : 0.f;
-    const float vx = vi.x - vj.x, vy = vi.y - vj.y, vz = vi.z - vj.z;
-    const float mu = fmaf(vx, dx, fmaf(vy, dy, vz * dz)) * rinv;
-    // viscosity only on approach (mu < 0): branch-free, Pi = 0 otherwise
-    const float muc = fminf(mu, 0.f);
-    const float vsig_ij = ti.z + tj.z - 3.f * muc;
-    const float Pi = -alpha * vsig_ij * muc * (0.5f * (ti.w + tj.w)) * __fdividef(1.f, ti.x + tj.x);
-    const float dWbar = 0.5f * (dWi + dWj);
-    const float mj = vj.w;
-    const float sc = mj * fmaf(ti.y, dWi, fmaf(tj.y, dWj, Pi * dWbar)) * rinv;
-    f.x = fmaf(-sc, dx, f.x);
-    f.y = fmaf(-sc, dy, f.y);
-    f.z = fmaf(-sc, dz, f.z);
-    f.u = fmaf(mj * mu, fmaf(ti.y, dWi, 0.5f * Pi * dWbar), f.u);
-    f.v = fmaxf(f.v, vsig_ij);
-}
-
 // MODE: 0 = uniform grid, 1 = adaptive cells (leaf lists), 2 = uniform grid with the
 // per-axis sweep (SPH_FLAG_AXIS_SWEEP)
 template <int TW, bool HASH, int MODE>
 __global__ void __launch_bounds__(kPairThreads, kDensityBlocks) k_density(DensityArgs a)
 {
+    if (a.run_if && (*a.run_if & 1ull) == 0ull) return;  // the sums over the lists ran instead
     constexpr bool LIST = MODE == 1, SWEEP = MODE == 2;
     constexpr int TPW = 32 / TW;
     constexpr int B = kBatchD;
@@ -971,7 +749,7 @@ struct ForceArgs {
 template <int TW, int MODE>
 __global__ void __launch_bounds__(kPairThreads, MODE == 1 ? kForceBlocks : kForceBlocksU) k_force(ForceArgs a)
 {
-    if (a.run_if && *a.run_if == 0ull) return;  // the symmetric pass ran instead
+    if (a.run_if && *a.run_if == 0ull) return;  // the symmetric pass, or the list sums, ran instead
     constexpr bool LIST = MODE == 1, SWEEP = MODE == 2;
     constexpr int TPW = 32 / TW;
     constexpr int B = kBatchF;
@@ -1983,7 +1761,7 @@ int compact_active_tiles(sph_ctx *ctx)
     return SPH_OK;
 }
 
-int run_density_pass(sph_ctx *ctx, sph_particles *parts, bool last_pass, bool active_list)
+int run_density_pass(sph_ctx *ctx, sph_particles *parts, bool last_pass, bool active_list, bool if_no_lists)
 {
     DensityArgs a{};  // every field not set below is null / zero
     a.pos4 = ctx->pos4;
@@ -2029,6 +1807,7 @@ int run_density_pass(sph_ctx *ctx, sph_particles *parts, bool last_pass, bool ac
     a.gamma = ctx->p.gamma;
     a.use_balsara = ctx->p.use_balsara;
     a.last_pass = last_pass ? 1 : 0;
+    a.run_if = if_no_lists ? ctx->counters + C_STALE : nullptr;
     int rc = smem_optin(ctx);
     if (rc) return rc;
     const int g = pair_grid(ctx, kDensityBlocks);
@@ -2051,12 +1830,12 @@ int run_density_pass(sph_ctx *ctx, sph_particles *parts, bool last_pass, bool ac
 #undef SPH_LAUNCH_D
     timer_end(ctx, end);
     SPH_LAUNCH(ctx, "density kernel");
-    ctx->st.density_passes++;
+    if (!if_no_lists) ctx->st.density_passes++;
     return SPH_OK;
 }
 
 // active_list: the tiles compacted from ctx->active (individual time-steps)
-int run_force_pass(sph_ctx *ctx, sph_particles *parts, bool active_list)
+int run_force_pass(sph_ctx *ctx, sph_particles *parts, bool active_list, bool if_no_lists)
 {
     ForceArgs a{};
     a.pos4 = ctx->pos4;
@@ -2093,7 +1872,8 @@ int run_force_pass(sph_ctx *ctx, sph_particles *parts, bool active_list)
     const int g = pair_grid(ctx, ctx->adaptive ? kForceBlocks : kForceBlocksU);
     // symmetric variant (uniform grid, every target, radius-1 reach): the gather
     // kernel below then runs only if some cell needs the radius-2 stencil
-    const bool sym = ctx->sym_force && !ctx->adaptive && !a.fmask && !a.axis && !active_list &&
+    if (if_no_lists) a.run_if = ctx->counters + C_FOVF;
+    const bool sym = !if_no_lists && ctx->sym_force && !ctx->adaptive && !a.fmask && !a.axis && !active_list &&
                      ctx->n < ((int64_t)1 << 27);
     if (sym) {
         rc = ensure_sym(ctx);
@@ -2163,7 +1943,7 @@ int run_force_pass(sph_ctx *ctx, sph_particles *parts, bool active_list)
             parts->dudt, parts->vsig);
         SPH_LAUNCH(ctx, "symmetric force sums");
     }
-    ctx->st.force_passes++;
+    if (!if_no_lists) ctx->st.force_passes++;
     return SPH_OK;
 }
 

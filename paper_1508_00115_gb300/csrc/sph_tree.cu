@@ -655,7 +655,8 @@ template <bool COUNT>
 __device__ int leaf_pairs(int l, const int *__restrict__ leaf_node, const TreeNode *__restrict__ nodes,
                           const int *__restrict__ top_node, const int *__restrict__ node_leaf,
                           const double *__restrict__ leaf_cen, const BoxDev *__restrict__ bxs, int nb, double box,
-                          float4 *__restrict__ out, float *__restrict__ scale_out)
+                          const int2 *__restrict__ leaf_rng, float4 *__restrict__ out, int *__restrict__ out_slot,
+                          float *__restrict__ scale_out)
 {
     const TreeNode A = nodes[leaf_node[l]];
     const BoxDev g = bxs[nb == 1 ? 0 : tbox_of_cell(A.top, bxs, nb)];
@@ -699,6 +700,7 @@ __device__ int leaf_pairs(int l, const int *__restrict__ leaf_node, const TreeNo
                     const double sx = leaf_cen[3 * b] + kx * box - cAx, sy = leaf_cen[3 * b + 1] + ky * box - cAy,
                                  sz = leaf_cen[3 * b + 2] + kz * box - cAz;
                     out[cnt] = make_float4((float)sx, (float)sy, (float)sz, __int_as_float(b));
+                    out_slot[cnt] = leaf_rng[b].x;
                     // coordinates met in this pair's FP32 arithmetic are below
                     // |p_i| + |p_j| + |shift| <= (sides of both leaves + shift)
                     const double m = fmax(fabs(sx), fmax(fabs(sy), fabs(sz)));
@@ -725,7 +727,7 @@ __global__ void k_pairs_count(int nl_h, const int *__restrict__ nlp, const unsig
     const int nl = nlp ? *nlp : nl_h;
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += gridDim.x * blockDim.x)
         cnt[l] = (uint32_t)leaf_pairs<true>(l, leaf_node, nodes, top_node, node_leaf, leaf_cen, bxs, nb, box, nullptr,
-                                            nullptr);
+                                            nullptr, nullptr, nullptr);
 }
 
 // (device count: runs only when *ovf reports an overflowed warp walk and *err holds
@@ -735,13 +737,15 @@ __global__ void k_pairs_fill(int nl_h, const int *__restrict__ nlp, const unsign
                              const TreeNode *__restrict__ nodes, const int *__restrict__ top_node,
                              const int *__restrict__ node_leaf, const double *__restrict__ leaf_cen,
                              const BoxDev *__restrict__ bxs, int nb, double box, const uint32_t *__restrict__ off,
-                             float4 *__restrict__ list, float *__restrict__ scale)
+                             const int2 *__restrict__ leaf_rng, float4 *__restrict__ list, int *__restrict__ list_slot,
+                             float *__restrict__ scale)
 {
     if (ovf && *ovf == 0ull) return;
     if (err && *err) return;
     const int nl = nlp ? *nlp : nl_h;
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += gridDim.x * blockDim.x)
-        leaf_pairs<false>(l, leaf_node, nodes, top_node, node_leaf, leaf_cen, bxs, nb, box, list + off[l], scale + l);
+        leaf_pairs<false>(l, leaf_node, nodes, top_node, node_leaf, leaf_cen, bxs, nb, box, leaf_rng,
+                          list + off[l], list_slot + off[l], scale + l);
 }
 
 // The same lists built by one warp per leaf: the warp pops up to 32 (node, image)
@@ -768,6 +772,8 @@ struct WalkArgs {
     double box;
     const uint32_t *__restrict__ off;  // fill: first entry of every leaf
     float4 *__restrict__ list;         // fill: entries
+    int *__restrict__ list_slot;       // fill: first slot of every entry's leaf
+    const int2 *__restrict__ leaf_rng;
     float *__restrict__ scale;         // fill: coordinate scale per leaf
     uint32_t *__restrict__ cnt;        // count: entries per leaf
     unsigned long long *overflow;
@@ -849,6 +855,7 @@ __device__ void walk_leaf(const WalkArgs &a, int l, int2 *st)
                          sz = a.leaf_cen[3 * b + 2] + kz * a.box - cAz;
             const float fx = (float)sx, fy = (float)sy, fz = (float)sz;
             a.list[base + cnt + __popc(eb & lt)] = make_float4(fx, fy, fz, __int_as_float(b));
+            a.list_slot[base + cnt + __popc(eb & lt)] = a.leaf_rng[b].x;
             // coordinates met in this pair's FP32 arithmetic stay below the two leaf
             // sides plus the offset
             const float m = fmaxf(fabsf(fx), fmaxf(fabsf(fy), fabsf(fz)));
@@ -1080,7 +1087,7 @@ static int build_tree_device(sph_ctx *ctx, sph_particles *parts)
     const unsigned gw = (unsigned)(7 * sms);  // 7 blocks of 2 walking warps (32 KB stacks) per SM
     WalkArgs wa{0,       nlp,           nullptr,          nullptr,     T.leaf_node,  T.nodes,
                 T.top_node, T.node_leaf, T.leaf_cen,    ctx->d_boxes, ctx->n_boxes, ctx->p.box_size,
-                T.list_off, T.list,      T.leaf_scale, T.list_off,   &dc->walk_ovf, &dc->walk_ticket[0]};
+                T.list_off, T.list,      T.list_slot, T.leaf_rng, T.leaf_scale, T.list_off,   &dc->walk_ovf, &dc->walk_ticket[0]};
     k_leaf_walk<true><<<gw, 32 * kWalkWarps, 0, ctx->stream>>>(wa);
     SPH_LAUNCH(ctx, "leaf walk count");
     k_pairs_count<<<gp, 128, 0, ctx->stream>>>(0, nlp, &dc->walk_ovf, T.leaf_node, T.nodes, T.top_node, T.node_leaf,
@@ -1100,7 +1107,7 @@ static int build_tree_device(sph_ctx *ctx, sph_particles *parts)
     SPH_LAUNCH(ctx, "leaf walk fill");
     k_pairs_fill<<<gp, 128, 0, ctx->stream>>>(0, nlp, &dc->walk_ovf, &dc->err, T.leaf_node, T.nodes, T.top_node,
                                               T.node_leaf, T.leaf_cen, ctx->d_boxes, ctx->n_boxes, ctx->p.box_size,
-                                              T.list_off, T.list, T.leaf_scale);
+                                              T.list_off, T.leaf_rng, T.list, T.list_slot, T.leaf_scale);
     SPH_LAUNCH(ctx, "pair fill");
     if ((rc = order_tiles(ctx, ctx->tiles, ctx->n_tiles))) return rc;
     ctx->built = true;
@@ -1140,7 +1147,7 @@ int tree_prepare_device(sph_ctx *ctx, uint64_t *sig)
         (rc = grow(ctx, T.leaf_lo, T.cap_leaf_lo, n + 1)) || (rc = grow(ctx, T.leaf_hi, T.cap_leaf_hi, n + 1)) ||
         (rc = grow(ctx, T.leaf_scale, T.cap_leaf_scale, n + 1)) ||
         (rc = grow(ctx, T.nact_leaf, T.cap_nact_leaf, n + 1)) || (rc = grow(ctx, T.list_off, T.cap_list_off, n + 2)) ||
-        (rc = grow(ctx, T.list, T.cap_list, list_need)))
+        (rc = grow(ctx, T.list, T.cap_list, list_need)) || (rc = grow(ctx, T.list_slot, T.cap_list_slot, list_need)))
         return rc;
     if (!T.dc) SPH_CUDA(ctx, cudaMalloc(&T.dc, sizeof(TreeCounts)));
     if (!T.hc) SPH_CUDA(ctx, cudaMallocHost(&T.hc, sizeof(TreeCounts)));
@@ -1151,7 +1158,7 @@ int tree_prepare_device(sph_ctx *ctx, uint64_t *sig)
     // (the sort's ping-pong pair in either order: captures may swap it)
     const void *ptrs[] = {std::min(ctx->keys64, ctx->keys64_alt), std::max(ctx->keys64, ctx->keys64_alt), T.leaf_of, T.node_at, T.tord, T.act_ord, T.top_node,
                           T.nodes, T.node_leaf, T.front, T.front2, T.bounds, T.nkids, T.leaf_node, T.leaf_rng,
-                          T.leaf_cen, T.leaf_h, T.leaf_scale, T.nact_leaf, T.list_off, T.list, T.dc,
+                          T.leaf_cen, T.leaf_h, T.leaf_scale, T.nact_leaf, T.list_off, T.list, T.list_slot, T.dc,
                           T.leaf_lo, T.leaf_hi};
     const int64_t caps[] = {capf, T.dev_cap_nodes, T.cap_list, T.dev_cap_list, ctx->leaf_max};
     uint64_t hsh = 1469598103934665603ull;
@@ -1362,7 +1369,7 @@ int build_tree(sph_ctx *ctx, sph_particles *parts)
         // neighbour lists: count, scan, fill (warp walks; one-thread walks if a warp's
         // stack overflowed)
         WalkArgs wa{nl, nullptr, nullptr, nullptr, T.leaf_node, T.nodes, T.top_node, T.node_leaf, T.leaf_cen, ctx->d_boxes, ctx->n_boxes,
-                    ctx->p.box_size, T.list_off, T.list, T.leaf_scale, T.list_off, ctx->counters + C_WALKOVF, nullptr};
+                    ctx->p.box_size, T.list_off, T.list, T.list_slot, T.leaf_rng, T.leaf_scale, T.list_off, ctx->counters + C_WALKOVF, nullptr};
         SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_WALKOVF, 0, sizeof(unsigned long long), ctx->stream));
         k_leaf_walk<true><<<nblk(nl, kWalkWarps), 32 * kWalkWarps, 0, ctx->stream>>>(wa);
         SPH_LAUNCH(ctx, "leaf walk count");
@@ -1400,15 +1407,18 @@ int build_tree(sph_ctx *ctx, sph_particles *parts)
         T.h_u32[7] = (uint32_t)ne;  // list_off[nl] = total (pinned source, copied in order)
         SPH_CUDA(ctx, cudaMemcpyAsync(T.list_off + nl, &T.h_u32[7], sizeof(uint32_t), cudaMemcpyHostToDevice,
                                       ctx->stream));
-        if ((rc = grow(ctx, T.list, T.cap_list, ne + 1))) return rc;
+        if ((rc = grow(ctx, T.list, T.cap_list, ne + 1)) || (rc = grow(ctx, T.list_slot, T.cap_list_slot, ne + 1)))
+            return rc;
         if (warp_walk) {
             wa.list = T.list;
+            wa.list_slot = T.list_slot;
             k_leaf_walk<false><<<nblk(nl, kWalkWarps), 32 * kWalkWarps, 0, ctx->stream>>>(wa);
             SPH_LAUNCH(ctx, "leaf walk fill");
         } else {
             k_pairs_fill<<<nblk(nl, 128), 128, 0, ctx->stream>>>(nl, nullptr, nullptr, nullptr, T.leaf_node, T.nodes, T.top_node, T.node_leaf,
                                                                 T.leaf_cen, ctx->d_boxes, ctx->n_boxes,
-                                                                ctx->p.box_size, T.list_off, T.list, T.leaf_scale);
+                                                                ctx->p.box_size, T.list_off, T.leaf_rng, T.list, T.list_slot,
+                                                                T.leaf_scale);
             SPH_LAUNCH(ctx, "pair fill");
         }
         if ((rc = order_tiles(ctx, ctx->tiles, ctx->n_tiles))) return rc;
@@ -1660,7 +1670,7 @@ void free_tree(sph_ctx *ctx)
     AdaptiveTree &T = ctx->tree;
     void *ptrs[] = {ctx->keys64, ctx->keys64_alt, T.leaf_of, T.tord, T.act_ord, T.nact_leaf, T.node_at, T.top_node, T.nodes, T.front, T.front2,
                     T.bounds, T.nkids, T.node_leaf, T.leaf_node, T.leaf_rng, T.leaf_cen, T.leaf_h, T.leaf_lo, T.leaf_hi,
-                    T.leaf_scale, T.list_off, T.list};
+                    T.leaf_scale, T.list_off, T.list, T.list_slot};
     for (void *p : ptrs) cudaFree(p);
     cudaFree(T.dc);
     cudaFreeHost(T.hc);

@@ -1,0 +1,90 @@
+"""Neighbour lists of the pair sums: one search serves the h iteration and the force
+pass as long as no h leaves its list radius (4 % beyond the h of the search).  The cases
+here start the second call from h that leave it: for a few particles (searched for one by
+one, with the targets whose lists miss them) and for all of them (searched again as a
+whole).  The bar is that of the other parity tests: neighbour sets exact."""
+import numpy as np
+import pytest
+
+from paper_1508_00115_gb300 import inputs
+
+from _gpu_util import check_density, check_force, oracle_state
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _second_call(d, flags, factor, share, **kw):
+    """Converge, scale `share` of the h by `factor`, and run build, density and force again."""
+    from paper_1508_00115_gb300 import binding
+    n = int(d["x"].size)
+    ctx = binding.Context(n, flags=flags | binding.SPH_FLAG_NGB_HASH, **kw)
+    parts = binding.Particles(d)
+    ctx.build_cells(parts)
+    ctx.density(parts)
+    ctx.force(parts)
+    pick = torch.as_tensor(np.random.default_rng(5).random(n) < share, device="cuda")
+    parts.t["h"][pick] *= factor
+    ctx.build_cells(parts)
+    ctx.density(parts)
+    ctx.force(parts)
+    g = parts.numpy()
+    g["perm"], g["ngb_hash"], g["stats"] = ctx.permutation(), ctx.ngb_hash(), ctx.stats()
+    return g
+
+
+@pytest.mark.parametrize("adaptive", [False, True])
+@pytest.mark.parametrize("factor,share", [(0.9, 0.01), (0.9, 1.0), (1.2, 1.0), (0.6, 0.3)])
+def test_h_leaving_its_list_radius(adaptive, factor, share):
+    from paper_1508_00115_gb300 import binding
+    if adaptive:
+        d = inputs.plummer_mix(6000, seed=31, n_halos=6)
+        flags = binding.SPH_FLAG_ADAPTIVE
+    else:
+        d = inputs.uniform(6000, seed=32)
+        flags = 0
+    d = inputs.random_velocities(d, 0.3, 33)
+    g = _second_call(d, flags, factor, share, cell_factor=1.5)
+    s = oracle_state(g)
+    check_density(g, s)
+    check_force(g, s)
+
+
+@pytest.mark.parametrize("n", [200, 257, 1031])
+@pytest.mark.parametrize("tw", [0, 16])
+def test_lists_of_small_sets(n, tw):
+    """Partial tiles and batches, the pages' edges, stencils that span the box."""
+    from paper_1508_00115_gb300 import binding
+    d = inputs.random_velocities(inputs.uniform(n, seed=n), 0.2, n + 1)
+    g = _second_call(d, binding.SPH_FLAG_ADAPTIVE, 0.97, 1.0, tile_width=tw, leaf_max=32)
+    s = oracle_state(g)
+    check_density(g, s)
+    check_force(g, s)
+
+
+def test_lists_of_thousands_of_names():
+    """A dense clump of 3,000 inside the kernel of sparse particles: lists beyond the eight
+    lanes' share (the whole warp takes them) and over several chunks."""
+    from paper_1508_00115_gb300 import binding
+    rng = np.random.default_rng(9)
+    d = inputs.random_velocities(inputs.uniform(4000, seed=41), 0.2, 42)
+    for k in ("x", "y", "z"):
+        d[k][:3000] = 0.5 + 0.002 * (rng.random(3000) - 0.5)
+    g = _second_call(d, binding.SPH_FLAG_ADAPTIVE | binding.SPH_FLAG_TREE_H_GUESS, 0.98, 1.0)
+    assert g["n_ngb"].max() > 1000
+    s = oracle_state(g)
+    check_density(g, s)
+    check_force(g, s)
+
+
+def test_leaf_too_large_for_its_names():
+    """Groups of four coincident particles with leaves of at most two: a name holds the
+    indices 0 and 1 only, and the sums run without lists."""
+    from paper_1508_00115_gb300 import binding
+    d = inputs.random_velocities(inputs.uniform(2000, seed=51), 0.2, 52)
+    for k in ("x", "y", "z"):
+        d[k][:12] = np.repeat(d[k][:3], 4)
+    g = _second_call(d, binding.SPH_FLAG_ADAPTIVE, 1.0, 0.0, leaf_max=2)
+    s = oracle_state(g)
+    check_density(g, s)
+    check_force(g, s)
