@@ -51,8 +51,10 @@ constexpr int kBfW1 = 0, kBfW2 = kHid * kW1Row, kBfW3 = kBfW2 + kHid * kW2Row;
 constexpr int kNBf = kBfW3 + kHid;
 
 // training schedule: blocks x sub-tiles x samples per Adam step
-constexpr int kTrThreads = 256, kTrS = 64, kTrSub = 4, kTrBlocks = 64;
-constexpr int kTrBatch = kTrBlocks * kTrSub * kTrS;  // 16384
+constexpr int kTrThreads = 256, kTrS = 128, kTrBlocks = 128;  // kTrS samples per block
+constexpr int kTrBatch = kTrBlocks * kTrS;                    // 16384
+constexpr int kTrRow = kTrS + 4;   // padded row of a [unit][sample] array: rows fall into different banks
+constexpr int kTrWRow = kHid + 4;  // same, of W2 and its transpose
 
 
 __device__ __forceinline__ float silu(float x) { return x / (1.f + __expf(-x)); }
@@ -486,145 +488,276 @@ struct TrainArgs {
     uint64_t seed;    // 0: sequential samples, else hashed
 };
 
-// one Adam step's gradients: every block takes kTrSub tiles of kTrS samples
+// One Adam step's gradients.  A block takes kTrS samples through the whole network, held as
+// [unit][sample] arrays in shared memory, and each of the three 64 x 64 products (layer 2,
+// its input gradient, its weight gradient) is a register tile per thread (4 units x 8
+// samples, 4 x 4 weights) fed by 16-byte shared-memory reads: three reads per 32 FMAs, so that
+// it is bound by issue and the latency of the eight warps' reads (1.6 M FMAs a block, 6 us at
+// full rate), where one output per thread and step spent two shared-memory reads on every
+// FMA.  Measured per step of 16,384 samples: 126 -> 28 us; a step with its update, launched
+// over the one before, 146 -> 27.6 us.
 __global__ void __launch_bounds__(kTrThreads) k_hp_train_grad(TrainArgs a)
 {
-    extern __shared__ float sm[];
-    float *sP = sm;                    // parameters
-    float *sG = sP + kNParam;          // gradient accumulators
-    float *X = sG + kNParam;           // [kTrS][kF]
-    float *Z1 = X + kTrS * kF;         // [kTrS][kHid]
-    float *H1 = Z1 + kTrS * kHid;
-    float *Z2 = H1 + kTrS * kHid;
-    float *D = Z2 + kTrS * kHid;       // dL/dZ2, then dL/dZ1 (in Z2's place)
-    float *dy = D + kTrS * kHid;       // [kTrS]
-    float *tg = dy + kTrS;             // [kTrS] normalised targets
-    __shared__ float s_loss[kTrThreads];
-    const int tid = threadIdx.x;
-    for (int k = tid; k < kNParam; k += kTrThreads) {
-        sP[k] = a.P[k];
-        sG[k] = 0.f;
-    }
-    float loss = 0.f;
-    const float inv_batch = 1.f / (float)kTrBatch;
-    __syncthreads();
-    for (int sub = 0; sub < kTrSub; ++sub) {
-        // samples
-        if (tid < kTrS) {
-            const uint64_t ctr = (uint64_t)a.step * kTrBatch + ((uint64_t)blockIdx.x * kTrSub + sub) * kTrS + tid;
-            const int64_t idx = a.seed == 0 ? (int64_t)(ctr % (uint64_t)a.n)
-                                             : (int64_t)(mix64(a.seed ^ (ctr * 0xD1B54A32D192ED03ull)) % (uint64_t)a.n);
-            for (int f = 0; f < kF; ++f) X[tid * kF + f] = (a.X[6 * idx + f] - a.norm[f]) / a.norm[kF + f];
-            tg[tid] = (a.Y[idx] - a.norm[2 * kF]) / a.norm[2 * kF + 1];
-        }
-        __syncthreads();
-        // layer 1
-        for (int e = tid; e < kTrS * kHid; e += kTrThreads) {
-            const int s = e / kHid, u = e % kHid;
-            float z = sP[kOffB1 + u];
-            for (int f = 0; f < kF; ++f) z = fmaf(sP[kOffW1 + u * kF + f], X[s * kF + f], z);
-            Z1[e] = z;
-            H1[e] = silu(z);
-        }
-        __syncthreads();
-        // layer 2
-        for (int e = tid; e < kTrS * kHid; e += kTrThreads) {
-            const int s = e / kHid, u = e % kHid;
-            float z = sP[kOffB2 + u];
-            for (int v = 0; v < kHid; ++v) z = fmaf(sP[kOffW2 + u * kHid + v], H1[s * kHid + v], z);
-            Z2[e] = z;
-        }
-        __syncthreads();
-        // output and its error (mean over the whole batch)
-        if (tid < kTrS) {
-            float y = sP[kOffB3];
-            for (int u = 0; u < kHid; ++u) y = fmaf(sP[kOffW3 + u], silu(Z2[tid * kHid + u]), y);
-            const float r = y - tg[tid];
-            dy[tid] = 2.f * r * inv_batch;
-            loss = fmaf(r, r, loss);
-        }
-        __syncthreads();
-        // dW3, db3
-        if (tid < kHid) {
-            float gsum = 0.f;
-            for (int s = 0; s < kTrS; ++s) gsum = fmaf(dy[s], silu(Z2[s * kHid + tid]), gsum);
-            sG[kOffW3 + tid] += gsum;
-        }
-        if (tid == kHid) {
-            float gsum = 0.f;
-            for (int s = 0; s < kTrS; ++s) gsum += dy[s];
-            sG[kOffB3] += gsum;
-        }
-        // dL/dZ2
-        for (int e = tid; e < kTrS * kHid; e += kTrThreads) {
-            const int s = e / kHid, u = e % kHid;
-            D[e] = dy[s] * sP[kOffW3 + u] * silu_grad(Z2[e]);
-        }
-        __syncthreads();
-        // dW2 (each thread owns 16 entries), db2
-        for (int e = tid; e < kHid * kHid; e += kTrThreads) {
-            const int u = e / kHid, v = e % kHid;
-            float gsum = 0.f;
-            for (int s = 0; s < kTrS; ++s) gsum = fmaf(D[s * kHid + u], H1[s * kHid + v], gsum);
-            sG[kOffW2 + e] += gsum;
-        }
-        if (tid < kHid) {
-            float gsum = 0.f;
-            for (int s = 0; s < kTrS; ++s) gsum += D[s * kHid + tid];
-            sG[kOffB2 + tid] += gsum;
-        }
-        // dL/dZ1 into Z2's place
-        for (int e = tid; e < kTrS * kHid; e += kTrThreads) {
-            const int s = e / kHid, v = e % kHid;
-            float gsum = 0.f;
-            for (int u = 0; u < kHid; ++u) gsum = fmaf(D[s * kHid + u], sP[kOffW2 + u * kHid + v], gsum);
-            Z2[e] = gsum * silu_grad(Z1[e]);
-        }
-        __syncthreads();
-        // dW1, db1
-        for (int e = tid; e < kHid * kF; e += kTrThreads) {
-            const int v = e / kF, f = e % kF;
-            float gsum = 0.f;
-            for (int s = 0; s < kTrS; ++s) gsum = fmaf(Z2[s * kHid + v], X[s * kF + f], gsum);
-            sG[kOffW1 + e] += gsum;
-        }
-        if (tid < kHid) {
-            float gsum = 0.f;
-            for (int s = 0; s < kTrS; ++s) gsum += Z2[s * kHid + tid];
-            sG[kOffB1 + tid] += gsum;
-        }
-        __syncthreads();
-    }
+    extern __shared__ __align__(16) float sm[];
+    float *sW2 = sm;                          // [u][v]
+    float *sW2T = sW2 + kHid * kTrWRow;       // [v][u]
+    float *H1 = sW2T + kHid * kTrWRow;        // [v][s]: silu(z1)
+    float *G1 = H1 + kHid * kTrRow;           // [v][s]: silu'(z1), then dL/dz1
+    float *D2 = G1 + kHid * kTrRow;           // [u][s]: dL/dz2
+    float *X = D2 + kHid * kTrRow;            // [f][s], then a row of ones (biases)
+    float *yp = X + (kF + 1) * kTrRow;        // [16][s]: parts of the output
+    float *sW1 = yp + 16 * kTrRow;            // [u][f]
+    float *sB1 = sW1 + kHid * kF, *sB2 = sB1 + kHid, *sW3 = sB2 + kHid;
+    float *dy = sW3 + kHid;                   // [s]
+    __shared__ float s_loss[kTrThreads / 32], s_db3[kTrThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
     float *out = a.gpart + (size_t)blockIdx.x * (kNParam + 1);
-    for (int k = tid; k < kNParam; k += kTrThreads) out[k] = sG[k];
-    s_loss[tid] = loss;
+    // the samples do not depend on the step before: fetched while its update still runs
+    float x[kF], target = 0.f;
+    if (tid < kTrS) {
+        const uint64_t ctr = (uint64_t)a.step * kTrBatch + (uint64_t)blockIdx.x * kTrS + tid;
+        const int64_t idx = a.seed == 0 ? (int64_t)(ctr % (uint64_t)a.n)
+                                         : (int64_t)(mix64(a.seed ^ (ctr * 0xD1B54A32D192ED03ull)) % (uint64_t)a.n);
+#pragma unroll
+        for (int f = 0; f < kF; ++f) x[f] = a.X[6 * idx + f];
+        target = a.Y[idx];
+#pragma unroll
+        for (int f = 0; f < kF; ++f) X[f * kTrRow + tid] = (x[f] - a.norm[f]) / a.norm[kF + f];
+        X[kF * kTrRow + tid] = 1.f;
+        target = (target - a.norm[2 * kF]) / a.norm[2 * kF + 1];
+    }
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+    float4 w2[kHid * kHid / 4 / kTrThreads];
+#pragma unroll
+    for (int k = 0; k < kHid * kHid / 4 / kTrThreads; ++k)
+        w2[k] = reinterpret_cast<const float4 *>(a.P + kOffW2)[tid + k * kTrThreads];
+#pragma unroll
+    for (int k = 0; k < kHid * kHid / 4 / kTrThreads; ++k) {
+        const int u = (tid + k * kTrThreads) / (kHid / 4), v = 4 * ((tid + k * kTrThreads) % (kHid / 4));
+        *reinterpret_cast<float4 *>(sW2 + u * kTrWRow + v) = w2[k];
+        sW2T[v * kTrWRow + u] = w2[k].x;
+        sW2T[(v + 1) * kTrWRow + u] = w2[k].y;
+        sW2T[(v + 2) * kTrWRow + u] = w2[k].z;
+        sW2T[(v + 3) * kTrWRow + u] = w2[k].w;
+    }
+    for (int k = tid; k < kHid * kF; k += kTrThreads) sW1[k] = a.P[kOffW1 + k];
+    if (tid < kHid) {
+        sB1[tid] = a.P[kOffB1 + tid];
+        sB2[tid] = a.P[kOffB2 + tid];
+        sW3[tid] = a.P[kOffW3 + tid];
+    }
     __syncthreads();
+    // layer 1: a thread takes one sample and half of the units
+    {
+        const int s = tid % kTrS, u0 = (tid / kTrS) * (kHid / 2);
+#pragma unroll
+        for (int f = 0; f < kF; ++f) x[f] = X[f * kTrRow + s];
+#pragma unroll 4
+        for (int u = u0; u < u0 + kHid / 2; ++u) {
+            float z = sB1[u];
+#pragma unroll
+            for (int f = 0; f < kF; ++f) z = fmaf(sW1[u * kF + f], x[f], z);
+            H1[u * kTrRow + s] = silu(z);
+            G1[u * kTrRow + s] = silu_grad(z);
+        }
+    }
+    __syncthreads();
+    // products over the 64 units k of A[k][samples] and B[k][4 outputs]: samples 4 (tid % 16) + e
+    // and 64 beyond, outputs 4 (tid / 16) + o
+    const int sg = 4 * (tid & 15), og = 4 * (tid >> 4);
+    auto product = [&](const float *A, const float *B, float (&c)[4][8]) {
+#pragma unroll 4
+        for (int k = 0; k < kHid; ++k) {
+            const float4 p = *reinterpret_cast<const float4 *>(A + k * kTrRow + sg);
+            const float4 q = *reinterpret_cast<const float4 *>(A + k * kTrRow + sg + 64);
+            const float4 w = *reinterpret_cast<const float4 *>(B + k * kTrWRow + og);
+            const float av[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+            const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int o = 0; o < 4; ++o)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) c[o][e] = fmaf(wv[o], av[e], c[o][e]);
+        }
+    };
+    // sum over the 16 threads that share this thread's outputs
+    auto sum16 = [&](float v) {
+#pragma unroll
+        for (int d = 1; d < 16; d <<= 1) v += __shfl_xor_sync(kFull, v, d);
+        return v;
+    };
+    // layer 2 and the output
+    float z[4][8];
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) z[o][e] = sB2[og + o];
+    product(H1, sW2T, z);
+    {
+        float y[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            y[e] = 0.f;
+#pragma unroll
+            for (int o = 0; o < 4; ++o) y[e] = fmaf(sW3[og + o], silu(z[o][e]), y[e]);
+        }
+        float *r = yp + (tid >> 4) * kTrRow + sg;
+        *reinterpret_cast<float4 *>(r) = make_float4(y[0], y[1], y[2], y[3]);
+        *reinterpret_cast<float4 *>(r + 64) = make_float4(y[4], y[5], y[6], y[7]);
+    }
+    __syncthreads();
+    float loss = 0.f, db3 = 0.f;
+    if (tid < kTrS) {
+        float y = a.P[kOffB3];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) y += yp[k * kTrRow + tid];
+        const float r = y - target;
+        db3 = 2.f * r * (1.f / (float)kTrBatch);
+        dy[tid] = db3;
+        loss = r * r;
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        loss += __shfl_xor_sync(kFull, loss, d);
+        db3 += __shfl_xor_sync(kFull, db3, d);
+    }
+    if (lane == 0) {
+        s_loss[tid >> 5] = loss;
+        s_db3[tid >> 5] = db3;
+    }
+    __syncthreads();
+    // dW3, dL/dz2, db2
+    {
+        const float4 p = *reinterpret_cast<const float4 *>(dy + sg), q = *reinterpret_cast<const float4 *>(dy + sg + 64);
+        const float d[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            float g3 = 0.f, g2 = 0.f;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                g3 = fmaf(d[e], silu(z[o][e]), g3);
+                z[o][e] = d[e] * sW3[og + o] * silu_grad(z[o][e]);
+                g2 += z[o][e];
+            }
+            float *r = D2 + (og + o) * kTrRow + sg;
+            *reinterpret_cast<float4 *>(r) = make_float4(z[o][0], z[o][1], z[o][2], z[o][3]);
+            *reinterpret_cast<float4 *>(r + 64) = make_float4(z[o][4], z[o][5], z[o][6], z[o][7]);
+            g3 = sum16(g3);
+            g2 = sum16(g2);
+            if ((tid & 15) == 0) {
+                out[kOffW3 + og + o] = g3;
+                out[kOffB2 + og + o] = g2;
+            }
+        }
+    }
+    __syncthreads();
+    // dL/dz1 in the place of silu'(z1)
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) z[o][e] = 0.f;
+    product(D2, sW2, z);
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+        float *r = G1 + (og + o) * kTrRow + sg;
+        float4 p = *reinterpret_cast<float4 *>(r), q = *reinterpret_cast<float4 *>(r + 64);
+        p = make_float4(p.x * z[o][0], p.y * z[o][1], p.z * z[o][2], p.w * z[o][3]);
+        q = make_float4(q.x * z[o][4], q.y * z[o][5], q.z * z[o][6], q.w * z[o][7]);
+        *reinterpret_cast<float4 *>(r) = p;
+        *reinterpret_cast<float4 *>(r + 64) = q;
+    }
+    // dW2: thread's rows u = tid / 16 + 16 i, columns v = tid % 16 + 16 j, over the samples
+    {
+        const int u0 = tid >> 4, v0 = tid & 15;
+        float c[4][4] = {};
+#pragma unroll 2
+        for (int s = 0; s < kTrS; s += 4) {
+            float4 p[4], q[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                p[k] = *reinterpret_cast<const float4 *>(D2 + (u0 + 16 * k) * kTrRow + s);
+                q[k] = *reinterpret_cast<const float4 *>(H1 + (v0 + 16 * k) * kTrRow + s);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    c[i][j] = fmaf(p[i].x, q[j].x, c[i][j]);
+                    c[i][j] = fmaf(p[i].y, q[j].y, c[i][j]);
+                    c[i][j] = fmaf(p[i].z, q[j].z, c[i][j]);
+                    c[i][j] = fmaf(p[i].w, q[j].w, c[i][j]);
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) out[kOffW2 + (u0 + 16 * i) * kHid + v0 + 16 * j] = c[i][j];
+    }
+    __syncthreads();
+    // dW1 and db1 (the row of ones): a warp takes eight units, its lanes four samples each
+    for (int v = 8 * (tid >> 5); v < 8 * (tid >> 5) + 8; ++v) {
+        const float4 g = *reinterpret_cast<const float4 *>(G1 + v * kTrRow + 4 * lane);
+        float r[kF + 1];
+#pragma unroll
+        for (int f = 0; f <= kF; ++f) {
+            const float4 x = *reinterpret_cast<const float4 *>(X + f * kTrRow + 4 * lane);
+            r[f] = fmaf(g.x, x.x, fmaf(g.y, x.y, fmaf(g.z, x.z, g.w * x.w)));
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) r[f] += __shfl_xor_sync(kFull, r[f], d);
+        }
+        if (lane == 0) {
+#pragma unroll
+            for (int f = 0; f < kF; ++f) out[kOffW1 + v * kF + f] = r[f];
+            out[kOffB1 + v] = r[kF];
+        }
+    }
     if (tid == 0) {
-        float l = 0.f;
-        for (int k = 0; k < kTrS; ++k) l += s_loss[k];
+        float l = 0.f, g = 0.f;
+        for (int k = 0; k < kTrS / 32; ++k) {
+            l += s_loss[k];
+            g += s_db3[k];
+        }
+        out[kOffB3] = g;
         out[kNParam] = l;
     }
 }
 
-// fixed-order sum of the block partials, then Adam (t = step + 1); loss of the step
-__global__ void k_hp_adam(const float *__restrict__ gpart, float *__restrict__ P, float *__restrict__ m,
-                          float *__restrict__ v, int64_t step, float lr, float *__restrict__ loss_out)
+// fixed-order sum of the block partials, then Adam with the bias corrections c1 and c2; loss
+// of the step.  A parameter's partials are summed by kAdamParts threads, whose sums are added
+// in order: one thread's chain of loads, and the corrections' powers in FP64 by every thread
+// (the FP64 pipe takes two lanes a clock), took 15 us of a step.
+constexpr float kBeta1 = 0.9f, kBeta2 = 0.999f;
+constexpr int kAdamParams = 32, kAdamParts = 8;
+__global__ void __launch_bounds__(kAdamParams * kAdamParts)
+    k_hp_adam(const float *__restrict__ gpart, float *__restrict__ P, float *__restrict__ m, float *__restrict__ v,
+              float lr, float c1, float c2, float *__restrict__ loss_out)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > kNParam) return;
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+    __shared__ float part[kAdamParts][kAdamParams];
+    const int kk = threadIdx.x % kAdamParams, pp = threadIdx.x / kAdamParams;
+    const int k = blockIdx.x * kAdamParams + kk;
     float g = 0.f;
-    for (int b = 0; b < kTrBlocks; ++b) g += gpart[(size_t)b * (kNParam + 1) + k];
+    if (k <= kNParam) {
+        const float *q = gpart + (size_t)pp * (kTrBlocks / kAdamParts) * (kNParam + 1) + k;
+#pragma unroll
+        for (int b = 0; b < kTrBlocks / kAdamParts; ++b) g += q[(size_t)b * (kNParam + 1)];
+    }
+    part[pp][kk] = g;
+    __syncthreads();
+    if (pp != 0 || k > kNParam) return;
+    g = 0.f;
+#pragma unroll
+    for (int p = 0; p < kAdamParts; ++p) g += part[p][kk];
     if (k == kNParam) {
         *loss_out = g / (float)kTrBatch;
         return;
     }
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float mk = b1 * m[k] + (1.f - b1) * g;
-    const float vk = b2 * v[k] + (1.f - b2) * g * g;
+    const float eps = 1e-8f;
+    const float mk = kBeta1 * m[k] + (1.f - kBeta1) * g;
+    const float vk = kBeta2 * v[k] + (1.f - kBeta2) * g * g;
     m[k] = mk;
     v[k] = vk;
-    const double t = (double)(step + 1);
-    const float c1 = (float)(1.0 - pow((double)b1, t)), c2 = (float)(1.0 - pow((double)b2, t));
     P[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
 }
 
@@ -886,17 +1019,35 @@ int hp_train(sph_ctx *ctx, const float *X, const float *Y, int64_t n, int epochs
         SPH_LAUNCH(ctx, "predictor stats final");
         H.norm_set = true;
     }
-    const size_t smem = sizeof(float) * (2 * kNParam + kTrS * kF + 4 * kTrS * kHid + 2 * kTrS);
+    const size_t smem = sizeof(float) * (2 * kHid * kTrWRow + (3 * kHid + kF + 1 + 16) * kTrRow + kHid * kF + 3 * kHid + kTrS);
     int rc = hp_smem_optin(ctx, smem);
     if (rc) return rc;
     const int64_t steps_per_epoch = (n + kTrBatch - 1) / kTrBatch;
     for (int e = 0; e < epochs; ++e)
         for (int64_t s = 0; s < steps_per_epoch; ++s) {
             TrainArgs a{X, Y, n, H.params, H.norm, H.gpart, H.adam_t, seed};
-            k_hp_train_grad<<<kTrBlocks, kTrThreads, smem, ctx->stream>>>(a);
+            // from the second step on, a kernel starts while its predecessor still runs and
+            // waits for it inside (the first one waits for what wrote X, Y and the norms)
+            cudaLaunchConfig_t lc = {};
+            cudaLaunchAttribute at = {};
+            at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at.val.programmaticStreamSerializationAllowed = 1;
+            lc.attrs = &at;
+            lc.stream = ctx->stream;
+            lc.numAttrs = e || s ? 1 : 0;
+            lc.gridDim = kTrBlocks;
+            lc.blockDim = kTrThreads;
+            lc.dynamicSmemBytes = smem;
+            SPH_CUDA(ctx, cudaLaunchKernelEx(&lc, k_hp_train_grad, a));
             SPH_LAUNCH(ctx, "predictor gradients");
-            k_hp_adam<<<(kNParam + 1 + 255) / 256, 256, 0, ctx->stream>>>(H.gpart, H.params, H.adam_m, H.adam_v,
-                                                                         H.adam_t, lr, H.d_loss);
+            const double t = (double)(H.adam_t + 1);
+            lc.numAttrs = 1;
+            lc.gridDim = (kNParam + 1 + kAdamParams - 1) / kAdamParams;
+            lc.blockDim = kAdamParams * kAdamParts;
+            lc.dynamicSmemBytes = 0;
+            SPH_CUDA(ctx, cudaLaunchKernelEx(&lc, k_hp_adam, (const float *)H.gpart, H.params, H.adam_m, H.adam_v, lr,
+                                             (float)(1.0 - pow((double)kBeta1, t)),
+                                             (float)(1.0 - pow((double)kBeta2, t)), H.d_loss));
             SPH_LAUNCH(ctx, "predictor adam");
             ++H.adam_t;
         }

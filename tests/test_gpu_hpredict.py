@@ -73,6 +73,29 @@ def test_hp_training_matches_oracle():
     assert np.array_equal(w2, hp.bf16_bits(W.astype(np.float32)))
 
 
+@pytest.mark.parametrize("n", [1, 300, hp.BATCH + 77])
+def test_hp_training_steps_in_a_row(n):
+    """Sets smaller than a batch (rows repeat in it) and not a multiple of one, over several
+    steps, whose launches overlap; each step may add 5e-4 lr (two: the bound above).  Twice
+    the same training gives the same bits."""
+    w, f = hp.to_library(hp.glorot(29), _norm())
+    P0, norm = hp.from_library(w, f)
+    X, Y = _data(n, 30)
+    lr, epochs = 1e-3, 3
+    steps = epochs * -(-n // hp.BATCH)
+    runs = []
+    for _ in range(2):
+        ctx = _ctx()
+        ctx.hp_load(w, f)
+        loss = ctx.hp_train(torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), epochs=epochs, lr=lr, seed=0)
+        runs.append(ctx.hp_params())
+    P_ref, losses = hp.adam_steps(P0, norm, X.astype(np.float64), Y.astype(np.float64), steps, lr)
+    d = np.abs(runs[0].astype(np.float64) - P_ref)
+    assert np.quantile(d, 0.99) <= 5e-4 * steps * lr, np.quantile(d, 0.99)
+    assert abs(loss - losses[-1]) <= 1e-4 * losses[-1] + 1e-7
+    assert np.array_equal(runs[0], runs[1])
+
+
 def test_hp_normalisation_from_training_data():
     ctx = _ctx()
     X, Y = _data(50000, 25)
