@@ -91,6 +91,32 @@ def test_gravity_clustered_matches_oracle_and_conserves_momentum():
     assert np.abs((m[:, None] * a).sum(axis=0)).max() <= 1e-6 * np.sum(m * np.linalg.norm(a, axis=1))
 
 
+@pytest.mark.parametrize("tw", [32, 16])
+@pytest.mark.parametrize("eps", [0.0, 0.004])
+def test_gravity_every_number_of_targets_and_sources(tw, eps):
+    """Cells of 0 to 40 particles in turn (every number of targets per tile and lane, sources
+    at every offset in a chunk) and one of 3,000 (several sums of a target's terms).  Jittered
+    lattices inside the cells keep unsoftened separations apart (the bar above)."""
+    nc, rng = 9, np.random.default_rng(17)
+    xyz = []
+    for c in range(nc ** 3):
+        k = 3000 if c == 400 else c % 41
+        side = int(np.ceil(k ** (1 / 3) - 1e-9))
+        at = rng.permutation(side ** 3)[:k] if k else np.zeros(0, int)
+        p = np.stack([at % side, at // side % side, at // side ** 2], axis=1) + 0.5 if k else np.zeros((0, 3))
+        p = (p + rng.uniform(-0.1, 0.1, p.shape)) / max(side, 1)
+        xyz.append((np.array([c % nc, c // nc % nc, c // nc ** 2]) + 0.02 + 0.96 * p) / nc)
+    xyz = np.concatenate(xyz)
+    n = len(xyz)
+    d = inputs.uniform(n, seed=18)
+    d["x"], d["y"], d["z"] = (np.ascontiguousarray(xyz[:, k]) for k in range(3))
+    d["m"] = rng.uniform(0.5, 2.0, n) / n
+    d["h"] = np.full(n, 0.1)
+    g, (o,), st = _gpu_gravity(d, eps=eps, tile_width=tw)
+    assert st["nc"] == nc
+    _compare(o, oracle.grav_p2p(_state(g), nc, eps=eps))
+
+
 def test_gravity_is_deterministic():
     d = _field(20000, 9, clustered=True, h0=0.08)
     _, outs, _ = _gpu_gravity(d, eps=0.002, runs=2)
