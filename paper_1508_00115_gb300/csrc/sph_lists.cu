@@ -913,7 +913,7 @@ __device__ __forceinline__ float near_one(float hinv, float L)
 
 // The names of a list (left of them from page on), taken by G lanes (q: the lane's place
 // among them), two each per step: f(name, valid) twice, then end of step g().  Every lane of the
-// warp calls it.
+// warp calls it; what a list's lanes add does not depend on the lists beside it.
 template <int G, class F, class E>
 __device__ __forceinline__ void walk_list(const SumArgs &a, int left, int page, int q, F f, E g)
 {
@@ -932,7 +932,7 @@ __device__ __forceinline__ void walk_list(const SumArgs &a, int left, int page, 
             const unsigned d1 = x + 3 * G + q < m ? __ldg(nm + x + 3 * G) : 0u;
             f(c0, x + q < m);
             f(c1, x + G + q < m);
-            g();
+            if (x < m) g();  // (a compensated sum may round again when it is given a zero)
             c0 = d0;
             c1 = d1;
         }
