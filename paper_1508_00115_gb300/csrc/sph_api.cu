@@ -83,7 +83,7 @@ static int alloc_particles(sph_ctx *c, int64_t cap)
 {
     free_particles(c);
     cap = std::max<int64_t>(cap, 1);
-    int64_t sort_tiles = (cap + 4095) / 4096;
+    const int64_t sort_tiles = std::max<int64_t>((cap + 4095) / 4096, 128);  // (kRsRowTiles short tiles)
     c->tile_cap = cap + cap / kMinTile + 64;
     SPH_CUDA(c, cudaMalloc(&c->pos4, sizeof(float4) * cap));
     SPH_CUDA(c, cudaMalloc(&c->vel4, sizeof(float4) * cap));

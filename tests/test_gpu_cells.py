@@ -1,0 +1,41 @@
+"""The cell build's sort and prefix sums at the edges of their tiles: permutation and keys
+equal a stable argsort of the keys of the input order, exactly."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1508_00115_gb300 import binding, inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,h", [(1, 0.2), (33, 0.3), (1023, 0.1), (1025, 0.05), (16385, 0.03), (131072, 0.02),
+                                 (131073, 0.02), (262145, 0.012), (524288, 0.3), (524289, 0.008)])
+def test_build_is_a_stable_sort_by_cell_and_octant(n, h):
+    d = inputs.uniform(n, seed=n)
+    d["h"] = np.full(n, h)
+    ctx = binding.Context(n)
+    parts = binding.Particles(d)
+    ctx.build_cells(parts)
+    nc = ctx.stats()["nc"]
+    pos = [oracle.wrap(d[k], 1.0) for k in ("x", "y", "z")]
+    cell = oracle.cell_keys(*pos, 1.0, nc).astype(np.int64)
+    idx = (cell % nc, (cell // nc) % nc, cell // (nc * nc))
+    octant = sum((p >= (i + 0.5) / nc).astype(np.int64) << b for b, (p, i) in enumerate(zip(pos, idx)))
+    perm = np.argsort(cell * 8 + octant, kind="stable")
+    assert np.array_equal(ctx.permutation(), perm)
+    assert np.array_equal(ctx.cell_keys(), cell[perm])
+    ctx.close()
+
+
+@pytest.mark.parametrize("n", [900, 20000])
+def test_adaptive_build_keeps_every_particle(n):
+    d = inputs.plummer_mix(n, seed=n, n_halos=3)
+    ctx = binding.Context(n, flags=binding.SPH_FLAG_ADAPTIVE)
+    parts = binding.Particles(d)
+    ctx.build_cells(parts)
+    perm = ctx.permutation()
+    assert np.array_equal(np.sort(perm), np.arange(n))
+    assert np.array_equal(parts.numpy()["x"], d["x"][perm])
+    ctx.close()
