@@ -17,37 +17,6 @@ constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanChunk = kScanThreads * kScanItems;
 
-__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v)
-{
-    int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t t = __shfl_up_sync(kFull, v, o);
-        if (lane >= o) v += t;
-    }
-    return v;
-}
-
-// Exclusive scan of one value per thread over the block; returns the block total.
-__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *sh_warp, uint32_t &total)
-{
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    uint32_t inc = warp_incl_scan(v);
-    if (lane == 31) sh_warp[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-        uint32_t t = lane < nw ? sh_warp[lane] : 0u;
-        uint32_t ti = warp_incl_scan(t);
-        if (lane < nw) sh_warp[lane] = ti - t;
-        if (lane == 31) sh_warp[32] = ti;
-    }
-    __syncthreads();
-    uint32_t r = sh_warp[w] + inc - v;
-    total = sh_warp[32];
-    __syncthreads();
-    return r;
-}
-
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t *__restrict__ in, int64_t n,
                                                               uint32_t *__restrict__ bsum)
 {

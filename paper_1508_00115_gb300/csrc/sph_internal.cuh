@@ -133,6 +133,7 @@ struct TreeCounts {
     unsigned long long list_total;
     unsigned long long walk_ovf;   // a warp's list walk overflowed its stack
     unsigned walk_ticket[2];       // leaf tickets of the counting and the filling walk
+    unsigned level_ticket;         // blocks of a level's kernel that are done
 };
 // TreeCounts.err bits: the nodes did not fit (some leaves stay above leaf_max, the
 // lists remain exact), the neighbour lists did not fit (the step did no pair work)
@@ -390,6 +391,38 @@ int cuda_fail(sph_ctx *ctx, cudaError_t e, const char *what);
         cudaError_t e_ = cudaGetLastError();                          \
         if (e_ != cudaSuccess) return sph::cuda_fail(ctx, e_, what);  \
     } while (0)
+
+// prefix sums over a warp and a block
+__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v)
+{
+    int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        uint32_t t = __shfl_up_sync(kFull, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
+// Exclusive scan of one value per thread over the block; returns the block total.
+__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *sh_warp, uint32_t &total)
+{
+    int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    uint32_t inc = warp_incl_scan(v);
+    if (lane == 31) sh_warp[w] = inc;
+    __syncthreads();
+    if (w == 0) {
+        uint32_t t = lane < nw ? sh_warp[lane] : 0u;
+        uint32_t ti = warp_incl_scan(t);
+        if (lane < nw) sh_warp[lane] = ti - t;
+        if (lane == 31) sh_warp[32] = ti;
+    }
+    __syncthreads();
+    uint32_t r = sh_warp[w] + inc - v;
+    total = sh_warp[32];
+    __syncthreads();
+    return r;
+}
 
 // timing
 void timer_begin(sph_ctx *ctx, int kind, cudaEvent_t *out_end);

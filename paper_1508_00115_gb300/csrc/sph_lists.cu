@@ -932,10 +932,13 @@ __device__ __forceinline__ void walk_list(const SumArgs &a, int left, int page, 
             const unsigned d1 = x + 3 * G + q < m ? __ldg(nm + x + 3 * G) : 0u;
             f(c0, x + q < m);
             f(c1, x + G + q < m);
-            if (x < m) g();  // (a compensated sum may round again when it is given a zero)
+            g();
             c0 = d0;
             c1 = d1;
         }
+        // (lists that end their chunk before the longest beside them have been given zeros, which
+        // may round a compensated sum again, once: now each of them has been)
+        g();
         left -= m;
         page = nxt;
     }

@@ -147,19 +147,95 @@ __global__ void k_roots(const int *__restrict__ cs, int64_t ntop, const uint32_t
     t.level = 0;
     t.prefix = 0;
     t.parent = -1;
+    t.hmax = 0.f;
     nodes[id] = t;
     top_node[c] = id;
     front[id] = id;
 }
 
-// Refinement decision of every frontier node (one thread per node): a node is split
-// while it holds more than leaf_max particles (down to the Morton resolution); its
+// Refinement decision of a node by eight lanes (all lanes of the warp call it): a node is
+// split while it holds more than leaf_max particles (down to the Morton resolution); its
 // non-empty octants' particle ranges come from binary searches on the next Morton
-// digit.  Octants are joined along the Morton order into halves (4 octants, a slab)
-// or quarters (2 octants, a bar) of the node while the part holds at most leaf_max
-// particles (a leaf spanning several octants keeps its parent's cube), so that a node
-// just above leaf_max gives two to four full leaves instead of up to eight sparse
-// ones.  Word 9 of a node's bounds marks the octants that start a child.
+// digit, one per lane (one thread doing all seven waited for them one after another: 10 to
+// 12 us per level, where k_tree_level takes 5 with all it does).  Octants are joined along the Morton order
+// into halves (4 octants, a slab) or quarters (2 octants, a bar) of the node while the part
+// holds at most leaf_max particles (a leaf spanning several octants keeps its parent's
+// cube), so that a node just above leaf_max gives two to four full leaves instead of up to
+// eight sparse ones.  Word 9 of a node's bounds marks the octants that start a child.
+// Returns the child count.
+__device__ __forceinline__ int split_node(int lo, int hi, int level, int leaf_max, const uint64_t *__restrict__ keys,
+                                          int *__restrict__ out)
+{
+    const int l = (int)(threadIdx.x & 7);
+    const bool split = hi - lo > leaf_max && level < kMortonBits;
+    // octant l starts at the first slot whose next Morton digit is >= l
+    int x = lo;
+    if (split && l > 0) {
+        const int sh = 3 * (kMortonBits - 1 - level);
+        int y = hi;
+        while (x < y) {
+            const int mid = (x + y) >> 1;
+            if ((int)((keys[mid] >> sh) & 7u) < l) x = mid + 1;
+            else y = mid;
+        }
+    }
+    __syncwarp();
+    int b[9];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) b[k] = __shfl_sync(kFull, x, k, 8);
+    b[8] = hi;
+    if (!split) return 0;
+    // children: a half of the cube (octants 4h .. 4h + 3) if it holds at most
+    // leaf_max particles, else its quarters (octant pairs) that do, else octants
+    int some = 0;  // non-empty octants
+#pragma unroll
+    for (int k = 0; k < 8; ++k) some |= b[k + 1] > b[k] ? 1 << k : 0;
+    auto first_in = [&](int mask) { return (some & mask) & -(some & mask); };  // first non-empty octant of them
+    int starts = 0;
+#pragma unroll
+    for (int q0 = 0; q0 < 8; q0 += 4) {
+        if (b[q0 + 4] - b[q0] <= leaf_max) {
+            starts |= first_in(15 << q0);
+            continue;
+        }
+#pragma unroll
+        for (int p0 = q0; p0 < q0 + 4; p0 += 2)
+            starts |= b[p0 + 2] - b[p0] <= leaf_max ? first_in(3 << p0) : some & (3 << p0);
+    }
+    out[l] = x;
+    if (l < 2) out[8 + l] = l ? starts : hi;
+    return __popc(starts);
+}
+
+// the j-th child of a split node
+__device__ __forceinline__ TreeNode child_node(const TreeNode &t, int id, const int *b, int starts, int j)
+{
+    int k = 0, e;
+    for (int m = starts; j > 0; --j) m &= m - 1, starts = m;
+    k = __ffs(starts) - 1;
+    starts &= starts - 1;
+    // the child runs from octant k up to the next starting octant
+    e = starts ? __ffs(starts) - 1 : 8;
+    int octants = 1;
+    for (int f = k + 1; f < e; ++f) octants += b[f + 1] > b[f] ? 1 : 0;
+    TreeNode ch;
+    ch.lo = b[k];
+    ch.hi = b[e];
+    ch.child = -1;
+    ch.nchild = 0;
+    ch.top = t.top;
+    if (octants == 1) {  // one octant: its own cube
+        ch.level = t.level + 1;
+        ch.prefix = (t.prefix << 3) | (uint64_t)k;
+    } else {  // joined octants: the parent's cube
+        ch.level = t.level;
+        ch.prefix = t.prefix;
+    }
+    ch.parent = id;
+    ch.hmax = 0.f;  // (zero bits: k_node_climb counts the children there first)
+    return ch;
+}
+
 // (Sizes: the host count, or -- builds inside captured steps -- the level's node range
 // lvl[0] .. lvl[1] on the device, the kernel then covering cap entries and writing
 // zero counts past the frontier.)
@@ -168,59 +244,119 @@ __global__ void k_node_split(const int *__restrict__ front, int nfront_h, const 
                              int *__restrict__ bounds, uint32_t *__restrict__ nkids)
 {
     const int nfront = lvl ? lvl[1] - lvl[0] : nfront_h;
-    const int end = lvl ? cap : nfront;
-    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < end; w += gridDim.x * blockDim.x) {
-        if (w >= nfront) {
-            nkids[w] = 0u;
-            continue;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    for (int w0 = tid >> 5 << 2; w0 < nfront; w0 += nt >> 5 << 2) {
+        const int w = w0 + ((int)(threadIdx.x & 31) >> 3);
+        int lo = 0, hi = 0, level = 0;
+        if (w < nfront) {
+            const TreeNode &t = nodes[front[w]];
+            lo = t.lo;
+            hi = t.hi;
+            level = t.level;
         }
-        const TreeNode t = nodes[front[w]];
-        const bool split = (t.hi - t.lo) > leaf_max && t.level < kMortonBits;
-        int cnt = 0;
-        if (split) {
-            // child boundaries: first slot whose next Morton digit is >= k (k = 1..7)
-            const int sh = 3 * (kMortonBits - 1 - t.level);
-            int b[9];
-            b[0] = t.lo;
-            b[8] = t.hi;
-            for (int k = 1; k < 8; ++k) {
-                int lo = b[k - 1], hi = t.hi;  // digits are sorted: search from the previous bound
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if ((int)((keys[mid] >> sh) & 7u) < k) lo = mid + 1;
-                    else hi = mid;
-                }
-                b[k] = lo;
-            }
-            // children: a half of the cube (octants 4h .. 4h + 3) if it holds at most
-            // leaf_max particles, else its quarters (octant pairs) that do, else octants
-            int starts = 0;
-            auto first_in = [&](int k0, int k1) {  // first non-empty octant of [k0, k1)
-                int k = k0;
-                while (k < k1 && b[k + 1] == b[k]) ++k;
-                return k;
-            };
-            for (int q0 = 0; q0 < 8; q0 += 4) {
-                const int qn = b[q0 + 4] - b[q0];
-                if (qn <= leaf_max) {
-                    if (qn > 0) starts |= 1 << first_in(q0, q0 + 4);
-                    continue;
-                }
-                for (int p0 = q0; p0 < q0 + 4; p0 += 2) {
-                    const int pn = b[p0 + 2] - b[p0];
-                    if (pn <= leaf_max) {
-                        if (pn > 0) starts |= 1 << first_in(p0, p0 + 2);
-                        continue;
+        const int cnt = split_node(lo, hi, level, leaf_max, keys, bounds + (size_t)kBoundsW * w);
+        if (w < nfront && (threadIdx.x & 7) == 0) nkids[w] = (uint32_t)cnt;
+    }
+    if (lvl)
+        for (int w = nfront + tid; w < cap; w += nt) nkids[w] = 0u;
+}
+
+// A level of a device-sized build in one launch: the children of the frontier nodes of level
+// `level` (make; level -1: the roots, which are there), the refinement decision of each of
+// them, and, by the block that ends last, the prefix sum of their child counts and the
+// range of the next level (none if it does not fit).  Eight lanes per possible child.  The
+// frontiers are node ranges (children are numbered in frontier order), the counts and
+// bounds of one level are read while those of the next are written.
+struct LevelArgs {
+    TreeNode *nodes;
+    const uint64_t *keys;
+    const int *bounds;     // of level `level`
+    const uint32_t *off;   // prefix sums of its child counts
+    int *bounds_out;
+    uint32_t *kids_out;
+    TreeCounts *tc;
+    int level, leaf_max;
+    int64_t capf, cap_nodes;
+};
+
+__global__ void __launch_bounds__(256) k_tree_level(LevelArgs a)
+{
+    __shared__ uint32_t sh[33];
+    __shared__ bool last;
+    int *lb = a.tc->level_begin;
+    const int L = a.level + 1;  // the frontier that is split
+    const int base = lb[L], nnew = lb[L + 1] - base;
+    if (nnew == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) lb[L + 2] = lb[L + 1];
+        return;
+    }
+    const int lane = threadIdx.x & 31, l = lane & 7;
+    const bool make = a.level >= 0;
+    const int pbase = make ? lb[a.level] : 0;
+    const int npar = base - pbase, units = make ? 8 * npar : nnew;
+    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
+    for (int u0 = 4 * gw; u0 < units; u0 += 4 * nw) {
+        const int u = u0 + (lane >> 3);
+        int w = -1, lo = 0, hi = 0, level = 0;
+        if (make) {
+            const int f = u >> 3, j = u & 7;  // a warp's four units share the parent
+            const int first = (int)a.off[f], kids = (f + 1 < npar ? (int)a.off[f + 1] : nnew) - first;
+            if (j < kids) {
+                w = first + j;
+                const int *b = a.bounds + (size_t)kBoundsW * f;
+                const TreeNode ch = child_node(a.nodes[pbase + f], pbase + f, b, b[9], j);
+                if (l == 0) {
+                    a.nodes[base + w] = ch;
+                    if (j == 0) {
+                        a.nodes[pbase + f].child = base + first;
+                        a.nodes[pbase + f].nchild = kids;
                     }
-                    for (int k = p0; k < p0 + 2; ++k)
-                        if (b[k + 1] > b[k]) starts |= 1 << k;
                 }
+                lo = ch.lo;
+                hi = ch.hi;
+                level = ch.level;
             }
-            cnt = __popc(starts);
-            for (int k = 0; k < 9; ++k) bounds[kBoundsW * w + k] = b[k];
-            bounds[kBoundsW * w + 9] = starts;
+        } else if (u < units) {
+            w = u;
+            lo = a.nodes[u].lo;
+            hi = a.nodes[u].hi;
         }
-        nkids[w] = (uint32_t)cnt;
+        if (!__any_sync(kFull, w >= 0)) continue;
+        const int cnt = split_node(lo, hi, level, a.leaf_max, a.keys, a.bounds_out + (size_t)kBoundsW * max(w, 0));
+        if (w >= 0 && l == 0) a.kids_out[w] = (uint32_t)cnt;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&a.tc->level_ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    constexpr int kItems = 8;
+    uint32_t carry = 0;
+    for (int i0 = 0; i0 < nnew; i0 += 256 * kItems) {
+        const int i = i0 + (int)threadIdx.x * kItems;
+        uint32_t v[kItems], sum = 0;
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) {
+            v[k] = i + k < nnew ? __ldcg(a.kids_out + i + k) : 0u;
+            sum += v[k];
+        }
+        uint32_t tot, e = block_excl_scan(sum, sh, tot) + carry;
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) {
+            if (i + k < nnew) a.kids_out[i + k] = e;
+            e += v[k];
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) {
+        int64_t nnext = carry;
+        if (nnext > a.capf || lb[L + 1] + nnext > a.cap_nodes) {
+            a.tc->err |= kTreeErrNodes;
+            nnext = 0;
+        }
+        lb[L + 2] = (int)(lb[L + 1] + nnext);
+        a.tc->level_ticket = 0u;
     }
 }
 
@@ -275,11 +411,50 @@ __global__ void k_leaf_box(TreeNode *__restrict__ nodes, int n_nodes_h, const in
     }
 }
 
-// internal nodes of one level [first, last): union of their children's boxes and max h
-__global__ void k_merge_children(TreeNode *__restrict__ nodes, int first_h, int last_h, const int *__restrict__ lb,
-                                 int level)
+// Device-sized builds: the boxes of all internal nodes in one launch.  A thread climbs from
+// every leaf; at each node all but the last child's stop, and the last takes the union of
+// the children's boxes and their largest h (in any order: the same values).  Until then
+// a node's hmax word counts its children that are done.  A launch per level spent 14 x 2 us
+// and the gaps between them, mostly on empty levels.
+__global__ void k_node_climb(TreeNode *nodes, const int *__restrict__ np)
 {
-    const int first = lb ? lb[level] : first_h, last = lb ? lb[level + 1] : last_h;
+    const int n_nodes = *np;
+    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < n_nodes; w += gridDim.x * blockDim.x) {
+        if (nodes[w].child >= 0) continue;
+        int id = nodes[w].parent;
+        while (id >= 0) {
+            TreeNode *d = nodes + id;
+            const int first = d->child, kids = d->nchild;
+            __threadfence();
+            if (atomicAdd(reinterpret_cast<int *>(&d->hmax), 1) != kids - 1) break;
+            __threadfence();
+            float hm = 0.f, x0 = 1e30f, y0 = 1e30f, z0 = 1e30f, x1 = -1e30f, y1 = -1e30f, z1 = -1e30f;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {  // (all reads in flight: past the last child its own again)
+                const TreeNode *k = nodes + first + min(c, kids - 1);
+                hm = fmaxf(hm, __ldcg(&k->hmax));
+                x0 = fminf(x0, __ldcg(&k->bx0));
+                y0 = fminf(y0, __ldcg(&k->by0));
+                z0 = fminf(z0, __ldcg(&k->bz0));
+                x1 = fmaxf(x1, __ldcg(&k->bx1));
+                y1 = fmaxf(y1, __ldcg(&k->by1));
+                z1 = fmaxf(z1, __ldcg(&k->bz1));
+            }
+            d->hmax = hm;
+            d->bx0 = x0;
+            d->by0 = y0;
+            d->bz0 = z0;
+            d->bx1 = x1;
+            d->by1 = y1;
+            d->bz1 = z1;
+            id = d->parent;
+        }
+    }
+}
+
+// internal nodes of one level [first, last): union of their children's boxes and max h
+__global__ void k_merge_children(TreeNode *__restrict__ nodes, int first, int last)
+{
     for (int id = first + blockIdx.x * blockDim.x + threadIdx.x; id < last; id += gridDim.x * blockDim.x) {
         TreeNode t = nodes[id];
         if (t.child < 0) continue;
@@ -323,37 +498,14 @@ __global__ void k_make_children(const int *__restrict__ front, int nfront_h, Tre
         const int *b = bounds + kBoundsW * f;
         const int starts = b[9];
         TreeNode &t = nodes[id];
-        int c = 0;
-        for (int k = 0; k < 8; ++k) {
-            if (!((starts >> k) & 1)) continue;
-            // the child runs from octant k up to the next starting octant
-            int e = k + 1;
-            int octants = 1;
-            while (e < 8 && !((starts >> e) & 1)) {
-                octants += b[e + 1] > b[e] ? 1 : 0;
-                ++e;
-            }
-            TreeNode ch;
-            ch.lo = b[k];
-            ch.hi = b[e];
-            ch.child = -1;
-            ch.nchild = 0;
-            ch.top = t.top;
-            if (octants == 1) {  // one octant: its own cube
-                ch.level = t.level + 1;
-                ch.prefix = (t.prefix << 3) | (uint64_t)k;
-            } else {  // joined octants: the parent's cube
-                ch.level = t.level;
-                ch.prefix = t.prefix;
-            }
-            ch.parent = id;
+        const int kids = (int)(end - first);
+        for (int c = 0; c < kids; ++c) {
             const int cid = base + (int)first + c;
-            nodes[cid] = ch;
+            nodes[cid] = child_node(t, id, b, starts, c);
             next[first + c] = cid;
-            ++c;
         }
         t.child = base + (int)first;
-        t.nchild = c;
+        t.nchild = kids;
     }
 }
 
@@ -955,6 +1107,7 @@ __global__ void k_tree_begin(const int *__restrict__ cs, int64_t ntop, const uin
     tc->list_total = 0ull;
     tc->walk_ovf = 0ull;
     tc->walk_ticket[0] = tc->walk_ticket[1] = 0u;
+    tc->level_ticket = 0u;
 }
 
 // children of level L: lb[L + 2] = lb[L + 1] + their count (none if they do not fit)
@@ -994,6 +1147,11 @@ __global__ void k_list_check(TreeCounts *__restrict__ tc, int64_t cap_list, int 
         *n_tiles = 0;
     }
 }
+
+// up to this many possible frontier nodes a level is one launch, its counts summed by one
+// block (actual frontiers are a tenth of it): 14 levels of 52,000 particles 270 -> 75 us of
+// device time, and 15 launches instead of 70
+constexpr int64_t kFusedFront = 65536;
 
 static int sm_count(sph_ctx *ctx)
 {
@@ -1038,7 +1196,16 @@ static int build_tree_device(sph_ctx *ctx, sph_particles *parts)
     SPH_LAUNCH(ctx, "tree roots");
     int *cur = T.front, *nxt = T.front2;
     int *lb = dc->level_begin;
-    for (int level = 0; level < kMortonBits; ++level) {
+    // the counts and bounds of two levels side by side, in the room that host builds need
+    const bool fused = capf <= kFusedFront && 2 * (capf + 1) <= T.cap_nkids && 2 * kBoundsW * (capf + 1) <= T.cap_bounds;
+    for (int level = -1; fused && level < kMortonBits; ++level) {
+        const int64_t in = level & 1 ? 0 : capf + 1, out = capf + 1 - in;
+        LevelArgs la{T.nodes, ctx->keys64, T.bounds + kBoundsW * in, T.nkids + in, T.bounds + kBoundsW * out, T.nkids + out,
+                     dc, level, ctx->leaf_max, capf, T.dev_cap_nodes};
+        k_tree_level<<<(unsigned)(2 * sms), 256, 0, ctx->stream>>>(la);
+        SPH_LAUNCH(ctx, "tree level");
+    }
+    for (int level = 0; !fused && level < kMortonBits; ++level) {
         k_node_split<<<gp, 256, 0, ctx->stream>>>(cur, 0, lb + level, (int)capf + 1, T.nodes, ctx->keys64,
                                                   ctx->leaf_max, T.bounds, T.nkids);
         SPH_LAUNCH(ctx, "node split");
@@ -1053,10 +1220,8 @@ static int build_tree_device(sph_ctx *ctx, sph_particles *parts)
     k_leaf_box<<<gp, 256, 0, ctx->stream>>>(T.nodes, 0, n_nodes, parts->x, parts->y, parts->z, parts->h,
                                             ctx->d_boxes, ctx->n_boxes);
     SPH_LAUNCH(ctx, "leaf boxes");
-    for (int L = kMortonBits - 1; L >= 0; --L) {  // level kMortonBits holds leaves only
-        k_merge_children<<<gp, 256, 0, ctx->stream>>>(T.nodes, 0, 0, lb, L);
-        SPH_LAUNCH(ctx, "merge children");
-    }
+    k_node_climb<<<gp, 256, 0, ctx->stream>>>(T.nodes, n_nodes);
+    SPH_LAUNCH(ctx, "node boxes");
     // leaves in particle order
     SPH_CUDA(ctx, cudaMemsetAsync(ctx->keys, 0, sizeof(uint32_t) * n, ctx->stream));
     k_leaf_marks<<<gp, 256, 0, ctx->stream>>>(T.nodes, 0, n_nodes, ctx->keys, T.node_at);
@@ -1262,7 +1427,7 @@ int build_tree(sph_ctx *ctx, sph_particles *parts)
     int *cur = T.front, *nxt = T.front2;
     std::vector<int> level_begin(1, 0);  // nodes of level L: [level_begin[L], level_begin[L + 1])
     for (int level = 0; level <= kMortonBits && nfront > 0; ++level) {
-        k_node_split<<<nblk(nfront, 256), 256, 0, ctx->stream>>>(cur, nfront, nullptr, 0, T.nodes, ctx->keys64,
+        k_node_split<<<nblk(8 * (int64_t)nfront, 256), 256, 0, ctx->stream>>>(cur, nfront, nullptr, 0, T.nodes, ctx->keys64,
                                                                  ctx->leaf_max, T.bounds, T.nkids);
         SPH_LAUNCH(ctx, "node split");
         SPH_CUDA(ctx, cudaMemcpyAsync(&T.h_u32[1], T.nkids + (nfront - 1), sizeof(uint32_t), cudaMemcpyDeviceToHost,
@@ -1294,7 +1459,7 @@ int build_tree(sph_ctx *ctx, sph_particles *parts)
         for (int L = (int)level_begin.size() - 2; L >= 0; --L) {
             const int first = level_begin[L], last = level_begin[L + 1];
             if (last <= first) continue;
-            k_merge_children<<<nblk(last - first, 256), 256, 0, ctx->stream>>>(T.nodes, first, last, nullptr, 0);
+            k_merge_children<<<nblk(last - first, 256), 256, 0, ctx->stream>>>(T.nodes, first, last);
             SPH_LAUNCH(ctx, "merge children");
         }
         return SPH_OK;

@@ -39,3 +39,26 @@ def test_adaptive_build_keeps_every_particle(n):
     assert np.array_equal(np.sort(perm), np.arange(n))
     assert np.array_equal(parts.numpy()["x"], d["x"][perm])
     ctx.close()
+
+
+@pytest.mark.parametrize("n,leaf", [(900, 2), (3000, 8), (5000, 300), (120000, 8)])
+def test_device_sized_trees_step_like_host_built_ones(n, leaf):
+    """Captured steps build the tree a level per launch with its sizes on the device (beyond
+    65,536 possible frontier nodes in several), host steps with host reads: deep trees, trees
+    of roots only, joined octants.  Tolerances: test_gpu_adaptive.py."""
+    from test_gpu_adaptive import _RT_RHO, _RT_STEPS, _same_state
+    d = inputs.uniform(n, seed=n) if n < 1000 else inputs.plummer_mix(n, seed=n, n_halos=4)
+    d = inputs.random_velocities(d, 0.2, 3)
+    out = []
+    for captured in (False, True):
+        ctx = binding.Context(n, flags=binding.SPH_FLAG_ADAPTIVE, h_tol=1e-6, leaf_max=leaf, max_h_iter=60)
+        parts = binding.Particles(d)
+        if captured:
+            ctx.steps(parts, 2, 1e-7)
+            assert ctx.stats()["graph_steps"] == 2
+        else:
+            ctx.step(parts, 1e-7)
+            ctx.step(parts, 1e-7)
+        out.append((parts.numpy(), ctx.permutation()))
+        ctx.close()
+    _same_state(out[0][0], out[1][0], out[0][1], out[1][1], _RT_STEPS, _RT_RHO)
