@@ -28,7 +28,12 @@ namespace sph {
 constexpr int kCodes = 1024;      // hits of a batch written out at once
 constexpr int kListThreads = 256;
 constexpr int kSearchBlocks = 3;  // resident blocks per SM the kernels are compiled for
-constexpr int kSumBlocks = 3;
+// the sums wait for scattered reads: a lane has both names of a step in flight, and five blocks
+// of four warps leave it the registers for that (Sedov 2 M, 19 M in 512 boxes, ms per call: one
+// name after the other at 24 warps per SM 14.4, 160; both at 24 warps 14.7, 154; at 20 13.4,
+// 152; at 16 13.7, 158)
+constexpr int kSumThreads = 128;
+constexpr int kSumBlocks = 5;
 constexpr int kSearchF4 = 352 + 2 * kCodes / 16;  // float4 of shared memory per searching warp
 constexpr int kPage = 32;         // names per page
 constexpr int kSlotBits = 25;     // uniform grid: bits of a name that hold the slot
@@ -912,8 +917,16 @@ __device__ __forceinline__ float near_one(float hinv, float L)
 }
 
 // The names of a list (left of them from page on), taken by G lanes (q: the lane's place
-// among them), two each per step: f(name, valid) twice, then end of step g().  Every lane of the
+// among them), two each per step: f(names, valid), then end of step g().  Every lane of the
 // warp calls it; what a list's lanes add does not depend on the lists beside it.
+struct Two {
+    unsigned v[2];
+    __device__ __forceinline__ unsigned operator[](int k) const { return v[k]; }
+};
+struct TwoBool {
+    bool v[2];
+    __device__ __forceinline__ bool operator[](int k) const { return v[k]; }
+};
 template <int G, class F, class E>
 __device__ __forceinline__ void walk_list(const SumArgs &a, int left, int page, int q, F f, E g)
 {
@@ -930,8 +943,7 @@ __device__ __forceinline__ void walk_list(const SumArgs &a, int left, int page, 
         for (int x = 0; __any_sync(kFull, x < m); x += 2 * G) {
             const unsigned d0 = x + 2 * G + q < m ? __ldg(nm + x + 2 * G) : 0u;
             const unsigned d1 = x + 3 * G + q < m ? __ldg(nm + x + 3 * G) : 0u;
-            f(c0, x + q < m);
-            f(c1, x + G + q < m);
+            f(Two{{c0, c1}}, TwoBool{{x + q < m, x + G + q < m}});
             g();
             c0 = d0;
             c1 = d1;
@@ -968,36 +980,60 @@ __device__ __forceinline__ void density_row(const DensityListArgs &a, const floa
     float rb = 0.f, wb = 0.f;
     walk_list<G>(
         a.s, t.left, t.page, q,
-        [&](unsigned name, bool ok) {
-            float sx = 0.f, sy = 0.f, sz = 0.f;
-            const int j = ok ? name_slot<MODE>(a.s, name, t.e0, t.L, shift, sx, sy, sz) : t.i;
-            const float4 pj = __ldg(a.s.pos4 + j);
-            const float4 vj = __ldg(a.s.vel4 + j);
-            const float dx = pi.x - (pj.x + sx), dy = pi.y - (pj.y + sy), dz = pi.z - (pj.z + sz);
-            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            const float rinv = inv_sqrt(r2);
-            float qq = ok ? r2 * rinv * hinv : 2.f;  // (the terms vanish from q = 1 on)
-            bool in = qq < 1.f;
-            // inside the FP32 band (rare) the FP64 separation decides
-            if (fabsf(qq - 1.f) < band) {
-                in = band_decide(a.s.x, a.s.y, a.s.z, t.i, j, a.s.box, t.h, t.h) & 1u;
-                qq = in ? qq : 1.f;
+        [&](Two name, TwoBool ok) {
+            // (both sources' reads first, one rare branch for both)
+            int j[2];
+            float4 pj[2], vj[2];
+            float dx[2], dy[2], dz[2], rinv[2], qq[2];
+            bool in[2], near = false;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float sx = 0.f, sy = 0.f, sz = 0.f;
+                j[e] = ok[e] ? name_slot<MODE>(a.s, name[e], t.e0, t.L, shift, sx, sy, sz) : t.i;
+                pj[e] = __ldg(a.s.pos4 + j[e]);
+                vj[e] = __ldg(a.s.vel4 + j[e]);
+                dx[e] = sx;
+                dy[e] = sy;
+                dz[e] = sz;
             }
-            float w, dw;
-            spline_u(qq, w, dw);
-            hits += in ? 1 : 0;
-            if (HASH && in) hh += mix64((uint64_t)a.ids[j]);
-            const float mj = vj.w;
-            rb = fmaf(mj, w, rb);
-            wb += w;
-            sqdw = fmaf(qq, dw, sqdw);
-            drho = fmaf(mj, fmaf(qq, dw, 3.f * w), drho);
-            const float fr = mj * dw * rinv;
-            const float vx = vi.x - vj.x, vy = vi.y - vj.y, vz = vi.z - vj.z;
-            dv = fmaf(fr, fmaf(vx, dx, fmaf(vy, dy, vz * dz)), dv);
-            cx = fmaf(fr, fmaf(vy, dz, -vz * dy), cx);
-            cy = fmaf(fr, fmaf(vz, dx, -vx * dz), cy);
-            cz = fmaf(fr, fmaf(vx, dy, -vy * dx), cz);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                dx[e] = pi.x - (pj[e].x + dx[e]);
+                dy[e] = pi.y - (pj[e].y + dy[e]);
+                dz[e] = pi.z - (pj[e].z + dz[e]);
+                const float r2 = fmaf(dx[e], dx[e], fmaf(dy[e], dy[e], dz[e] * dz[e]));
+                rinv[e] = inv_sqrt(r2);
+                qq[e] = ok[e] ? r2 * rinv[e] * hinv : 2.f;  // (the terms vanish from q = 1 on)
+                in[e] = qq[e] < 1.f;
+                near |= fabsf(qq[e] - 1.f) < band;
+            }
+            // inside the FP32 band (rare) the FP64 separation decides
+            if (near) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+                    if (fabsf(qq[e] - 1.f) < band) {
+                        in[e] = band_decide(a.s.x, a.s.y, a.s.z, t.i, j[e], a.s.box, t.h, t.h) & 1u;
+                        qq[e] = in[e] ? qq[e] : 1.f;
+                    }
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float w, dw;
+                spline_u(qq[e], w, dw);
+                hits += in[e] ? 1 : 0;
+                if (HASH && in[e]) hh += mix64((uint64_t)a.ids[j[e]]);
+                const float mj = vj[e].w;
+                rb = fmaf(mj, w, rb);
+                wb += w;
+                sqdw = fmaf(qq[e], dw, sqdw);
+                drho = fmaf(mj, fmaf(qq[e], dw, 3.f * w), drho);
+                const float fr = mj * dw * rinv[e];
+                const float vx = vi.x - vj[e].x, vy = vi.y - vj[e].y, vz = vi.z - vj[e].z;
+                dv = fmaf(fr, fmaf(vx, dx[e], fmaf(vy, dy[e], vz * dz[e])), dv);
+                cx = fmaf(fr, fmaf(vy, dz[e], -vz * dy[e]), cx);
+                cy = fmaf(fr, fmaf(vz, dx[e], -vx * dz[e]), cy);
+                cz = fmaf(fr, fmaf(vx, dy[e], -vy * dx[e]), cz);
+            }
         },
         [&]() {
             kahan_add(rho_s, rho_c, rb);
@@ -1027,15 +1063,15 @@ __device__ __forceinline__ void density_row(const DensityListArgs &a, const floa
 }
 
 template <int MODE, bool HASH>
-__global__ void __launch_bounds__(kListThreads, kSumBlocks) k_density_l(DensityListArgs a)
+__global__ void __launch_bounds__(kSumThreads, kSumBlocks) k_density_l(DensityListArgs a)
 {
     if (a.s.counters[C_STALE] & 1ull) return;  // no lists: the kernels of sph_pairs.cu run
     if (a.s.run_if && *a.s.run_if == 0ull) return;
     constexpr bool LIST = MODE == 1;
     __shared__ float4 shift[LIST ? 1 : 125];
-    __shared__ float s_sum[kListThreads / 32][32][9];
-    __shared__ unsigned long long s_hash[HASH ? kListThreads / 32 : 1][32];
-    __shared__ uint8_t s_ord[kListThreads / 32][32];
+    __shared__ float s_sum[kSumThreads / 32][32][9];
+    __shared__ unsigned long long s_hash[HASH ? kSumThreads / 32 : 1][32];
+    __shared__ uint8_t s_ord[kSumThreads / 32][32];
     if (!LIST) load_shifts(shift);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int grp8 = lane >> 3, q = lane & 7;
@@ -1290,10 +1326,12 @@ __global__ void __launch_bounds__(256) k_mark_dirty(MarkArgs a)
         const float4 pi = a.s.pos4[i];
         const float hf = a.h[i];
         const float top = fmaf(hf, hf, 2.f * kBandK * hf * (hf + L));
-        walk_list<32>(a.s, a.s.cnt[i], a.s.head[i], lane, [&](unsigned name, bool ok) {
-            if (ok) {
+        walk_list<32>(a.s, a.s.cnt[i], a.s.head[i], lane, [&](Two name, TwoBool ok) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (!ok[e]) continue;
                 float sx, sy, sz;
-                const int j = name_slot<MODE>(a.s, name, e0, L, shift, sx, sy, sz);
+                const int j = name_slot<MODE>(a.s, name[e], e0, L, shift, sx, sy, sz);
                 const float4 pj = a.s.pos4[j];
                 const float dx = pi.x - (pj.x + sx), dy = pi.y - (pj.y + sy), dz = pi.z - (pj.z + sz);
                 const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
@@ -1331,41 +1369,67 @@ __device__ __forceinline__ int force_row(const ForceListArgs &a, const float4 *s
     ForceSum part;
     walk_list<G>(
         a.s, left, page, q,
-        [&](unsigned name, bool ok) {
-            float fx = 0.f, fy = 0.f, fz = 0.f;
-            const int j = ok ? name_slot<MODE>(a.s, name, e0, L, shift, fx, fy, fz) : i;
-            const float4 pj = __ldg(a.s.pos4 + j);
-            const float4 vj = __ldg(a.s.vel4 + j);
-            const float4 tj = __ldg(a.s.thermo4 + j);
-            const float dx = pi.x - (pj.x + fx), dy = pi.y - (pj.y + fy), dz = pi.z - (pj.z + fz);
-            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            const float rinv = inv_sqrt(r2);
-            const float r = ok ? r2 * rinv : 1e30f;
-            const float hjinv = inv(pj.w), hj2inv = hjinv * hjinv;
-            float qi = r * hinv, qj = r * hjinv;  // (a term vanishes from q = 1 on)
-            // inside the FP32 band of either (rare) the FP64 separation decides
-            if (fabsf(qi - 1.f) < band_i || fabsf(qj - 1.f) < near_one(hjinv, L)) {
-                const unsigned d = band_decide(a.s.x, a.s.y, a.s.z, i, j, a.s.box, hi, pj.w);
-                qi = (d & 1u) ? fminf(qi, 0.99999994f) : fmaxf(qi, 1.f);
-                qj = (d & 2u) ? fminf(qj, 0.99999994f) : fmaxf(qj, 1.f);
+        [&](Two name, TwoBool ok) {
+            // (both sources' reads first, one rare branch for both)
+            int j[2];
+            float4 pj[2], vj[2], tj[2];
+            float dx[2], dy[2], dz[2], rinv[2], hjinv[2], qi[2], qj[2];
+            bool near = false;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float fx = 0.f, fy = 0.f, fz = 0.f;
+                j[e] = ok[e] ? name_slot<MODE>(a.s, name[e], e0, L, shift, fx, fy, fz) : i;
+                pj[e] = __ldg(a.s.pos4 + j[e]);
+                vj[e] = __ldg(a.s.vel4 + j[e]);
+                tj[e] = __ldg(a.s.thermo4 + j[e]);
+                dx[e] = fx;
+                dy[e] = fy;
+                dz[e] = fz;
             }
-            const bool in = fminf(qi, qj) < 1.f;
-            hits += in ? 1 : 0;
-            // the pair term (force_term), without sigma; the pair (i, i), and coincident pairs,
-            // have no direction: 1/r = 0
-            const float Wi = spline_dw_u(qi) * hinv4, Wj = spline_dw_u(qj) * (hj2inv * hj2inv);
-            const float vx = vi.x - vj.x, vy = vi.y - vj.y, vz = vi.z - vj.z;
-            const float mu = fmaf(vx, dx, fmaf(vy, dy, vz * dz)) * rinv;
-            const float muc = fminf(mu, 0.f);
-            const float vsig = ti.z + tj.z - 3.f * muc;
-            const float Pi = alpha * vsig * muc * (ti.w + tj.w) * inv(ti.x + tj.x) * (Wi + Wj);
-            const float mj = vj.w;
-            const float sc = mj * fmaf(ti.y, Wi, fmaf(tj.y, Wj, Pi)) * rinv;
-            part.x = fmaf(-sc, dx, part.x);
-            part.y = fmaf(-sc, dy, part.y);
-            part.z = fmaf(-sc, dz, part.z);
-            part.u = fmaf(mj * mu, fmaf(ti.y, Wi, 0.5f * Pi), part.u);
-            if (in && rinv > 0.f) vs = fmaxf(vs, vsig);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                dx[e] = pi.x - (pj[e].x + dx[e]);
+                dy[e] = pi.y - (pj[e].y + dy[e]);
+                dz[e] = pi.z - (pj[e].z + dz[e]);
+                const float r2 = fmaf(dx[e], dx[e], fmaf(dy[e], dy[e], dz[e] * dz[e]));
+                rinv[e] = inv_sqrt(r2);
+                const float r = ok[e] ? r2 * rinv[e] : 1e30f;
+                hjinv[e] = inv(pj[e].w);
+                qi[e] = r * hinv;  // (a term vanishes from q = 1 on)
+                qj[e] = r * hjinv[e];
+                near |= fabsf(qi[e] - 1.f) < band_i || fabsf(qj[e] - 1.f) < near_one(hjinv[e], L);
+            }
+            // inside the FP32 band of either (rare) the FP64 separation decides
+            if (near) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+                    if (fabsf(qi[e] - 1.f) < band_i || fabsf(qj[e] - 1.f) < near_one(hjinv[e], L)) {
+                        const unsigned d = band_decide(a.s.x, a.s.y, a.s.z, i, j[e], a.s.box, hi, pj[e].w);
+                        qi[e] = (d & 1u) ? fminf(qi[e], 0.99999994f) : fmaxf(qi[e], 1.f);
+                        qj[e] = (d & 2u) ? fminf(qj[e], 0.99999994f) : fmaxf(qj[e], 1.f);
+                    }
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const bool in = fminf(qi[e], qj[e]) < 1.f;
+                hits += in ? 1 : 0;
+                // the pair term (force_term), without sigma; the pair (i, i), and coincident pairs,
+                // have no direction: 1/r = 0
+                const float hj2inv = hjinv[e] * hjinv[e];
+                const float Wi = spline_dw_u(qi[e]) * hinv4, Wj = spline_dw_u(qj[e]) * (hj2inv * hj2inv);
+                const float vx = vi.x - vj[e].x, vy = vi.y - vj[e].y, vz = vi.z - vj[e].z;
+                const float mu = fmaf(vx, dx[e], fmaf(vy, dy[e], vz * dz[e])) * rinv[e];
+                const float muc = fminf(mu, 0.f);
+                const float vsig = ti.z + tj[e].z - 3.f * muc;
+                const float Pi = alpha * vsig * muc * (ti.w + tj[e].w) * inv(ti.x + tj[e].x) * (Wi + Wj);
+                const float mj = vj[e].w;
+                const float sc = mj * fmaf(ti.y, Wi, fmaf(tj[e].y, Wj, Pi)) * rinv[e];
+                part.x = fmaf(-sc, dx[e], part.x);
+                part.y = fmaf(-sc, dy[e], part.y);
+                part.z = fmaf(-sc, dz[e], part.z);
+                part.u = fmaf(mj * mu, fmaf(ti.y, Wi, 0.5f * Pi), part.u);
+                if (in && rinv[e] > 0.f) vs = fmaxf(vs, vsig);
+            }
         },
         [&]() {
             kahan_add(sx_, sxc, part.x);
@@ -1389,12 +1453,12 @@ __device__ __forceinline__ int force_row(const ForceListArgs &a, const float4 *s
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kListThreads, kSumBlocks) k_force_l(ForceListArgs a)
+__global__ void __launch_bounds__(kSumThreads, kSumBlocks) k_force_l(ForceListArgs a)
 {
     if (a.s.counters[C_FOVF]) return;
     constexpr bool LIST = MODE == 1;
     __shared__ float4 shift[LIST ? 1 : 125];
-    __shared__ float s_sum[kListThreads / 32][32][5];
+    __shared__ float s_sum[kSumThreads / 32][32][5];
     if (!LIST) load_shifts(shift);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int grp8 = lane >> 3, q = lane & 7;
@@ -1533,13 +1597,13 @@ int ensure_lists(sph_ctx *ctx, int64_t pages)
     return SPH_OK;
 }
 
-static int list_grid(sph_ctx *ctx, int blocks_per_sm, int split = 1)
+static int list_grid(sph_ctx *ctx, int threads, int blocks_per_sm, int split = 1)
 {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
     if (sms <= 0) sms = 148;
     const int64_t cells = ctx->adaptive ? ctx->tree.n_leaves : ctx->grid.n_cells;
-    const int64_t want = ((int64_t)ctx->n / ctx->tile_w + cells) / (kListThreads / 32) + 1;
+    const int64_t want = ((int64_t)ctx->n / ctx->tile_w + cells) / (threads / 32) + 1;
     return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * blocks_per_sm, want * split));
 }
 
@@ -1564,7 +1628,7 @@ static int tile_split(sph_ctx *ctx)
 {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
-    const int64_t warps = (int64_t)(sms > 0 ? sms : 148) * kSumBlocks * (kListThreads / 32);
+    const int64_t warps = (int64_t)(sms > 0 ? sms : 148) * kSumBlocks * (kSumThreads / 32);
     int split = 1;
     while (split < 8 && ctx->n / 32 * split < 4 * warps) split *= 2;
     return split;
@@ -1665,7 +1729,7 @@ int run_search(sph_ctx *ctx, sph_particles *parts, int pass)
     a.grow = force ? 1.f : ctx->lists.grow;
     a.wbits = name_bits(ctx);
     a.force = force ? 1 : 0;
-    const int g = list_grid(ctx, kSearchBlocks);
+    const int g = list_grid(ctx, kListThreads, kSearchBlocks);
     cudaEvent_t end = nullptr;
     timer_begin(ctx, force ? 1 : 0, &end);
     if (ctx->adaptive) k_search<1><<<g, kListThreads, kSearchSmem, ctx->stream>>>(a);
@@ -1758,15 +1822,15 @@ int run_density_lists(sph_ctx *ctx, sph_particles *parts, int pass, int budget, 
     a.last_pass = last_pass ? 1 : 0;
     a.hold_cells = ctx->tree.device_sized ? 1 : 0;  // captured steps
     const bool hash = (ctx->p.flags & SPH_FLAG_NGB_HASH) != 0;
-    const int g = list_grid(ctx, kSumBlocks, a.s.split);
+    const int g = list_grid(ctx, kSumThreads, kSumBlocks, a.s.split);
     cudaEvent_t end = nullptr;
     timer_begin(ctx, 0, &end);
     if (ctx->adaptive) {
-        if (hash) k_density_l<1, true><<<g, kListThreads, 0, ctx->stream>>>(a);
-        else k_density_l<1, false><<<g, kListThreads, 0, ctx->stream>>>(a);
+        if (hash) k_density_l<1, true><<<g, kSumThreads, 0, ctx->stream>>>(a);
+        else k_density_l<1, false><<<g, kSumThreads, 0, ctx->stream>>>(a);
     } else {
-        if (hash) k_density_l<0, true><<<g, kListThreads, 0, ctx->stream>>>(a);
-        else k_density_l<0, false><<<g, kListThreads, 0, ctx->stream>>>(a);
+        if (hash) k_density_l<0, true><<<g, kSumThreads, 0, ctx->stream>>>(a);
+        else k_density_l<0, false><<<g, kSumThreads, 0, ctx->stream>>>(a);
     }
     timer_end(ctx, end);
     SPH_LAUNCH(ctx, "density sums");
@@ -1786,11 +1850,11 @@ int run_force_lists(sph_ctx *ctx, sph_particles *parts)
     a.vsig = parts->vsig;
     a.fmask = ctx->bin_mode ? ctx->bin_active : nullptr;
     a.alpha = ctx->p.alpha_visc;
-    const int g = list_grid(ctx, kSumBlocks, a.s.split);
+    const int g = list_grid(ctx, kSumThreads, kSumBlocks, a.s.split);
     cudaEvent_t end = nullptr;
     timer_begin(ctx, 1, &end);
-    if (ctx->adaptive) k_force_l<1><<<g, kListThreads, 0, ctx->stream>>>(a);
-    else k_force_l<0><<<g, kListThreads, 0, ctx->stream>>>(a);
+    if (ctx->adaptive) k_force_l<1><<<g, kSumThreads, 0, ctx->stream>>>(a);
+    else k_force_l<0><<<g, kSumThreads, 0, ctx->stream>>>(a);
     timer_end(ctx, end);
     SPH_LAUNCH(ctx, "force sums");
     ctx->st.force_passes++;
