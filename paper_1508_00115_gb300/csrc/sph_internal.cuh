@@ -479,7 +479,8 @@ bool lists_apply(const sph_ctx *ctx);
 int ensure_lists(sph_ctx *ctx, int64_t pages);  // (outside captures)
 void free_lists(sph_ctx *ctx);
 int lists_begin(sph_ctx *ctx, bool force);
-int run_search(sph_ctx *ctx, sph_particles *parts, int pass);
+unsigned list_few_rows(const sph_ctx *ctx);
+int run_search(sph_ctx *ctx, sph_particles *parts, int pass, bool all = false);  // pass -1: the force pass's
 int run_density_lists(sph_ctx *ctx, sph_particles *parts, int pass, int budget, bool last_pass);
 int run_mark(sph_ctx *ctx, sph_particles *parts);
 int run_force_lists(sph_ctx *ctx, sph_particles *parts);

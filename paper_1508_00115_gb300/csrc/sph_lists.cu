@@ -1522,7 +1522,7 @@ __global__ void __launch_bounds__(kSumThreads, kSumBlocks) k_force_l(ForceListAr
 
 // Targets up to which the search for single targets runs: beyond, staging the sources
 // of whole leaves (cells) is cheaper.
-static unsigned few_rows(const sph_ctx *ctx) { return (unsigned)std::max<int64_t>(32, ctx->n / 24); }
+unsigned list_few_rows(const sph_ctx *ctx) { return (unsigned)std::max<int64_t>(32, ctx->n / 24); }
 
 // Start of a density call's searches (or of the force pass's own, which starts the pool
 // again only where it will run): the pool, the flags, and the tickets and counts of every
@@ -1616,7 +1616,7 @@ static int name_bits(const sph_ctx *ctx)
 
 int lists_begin(sph_ctx *ctx, bool force)
 {
-    k_lists_begin<<<1, 32, 0, ctx->stream>>>(ctx->counters, force ? 1 : 0, few_rows(ctx));
+    k_lists_begin<<<1, 32, 0, ctx->stream>>>(ctx->counters, force ? 1 : 0, list_few_rows(ctx));
     SPH_LAUNCH(ctx, "list pool");
     return SPH_OK;
 }
@@ -1684,7 +1684,7 @@ static int search_optin(sph_ctx *ctx)
 // Pass `pass` (below kListPasses) of a density call: lists for the active targets; a pass
 // after the first runs only if the one before left targets.  pass < 0: the force pass's own
 // search, at the converged h, where the lists of the density passes do not serve.
-int run_search(sph_ctx *ctx, sph_particles *parts, int pass)
+int run_search(sph_ctx *ctx, sph_particles *parts, int pass, bool all)
 {
     const ListPool &P = ctx->lists;
     const bool force = pass < 0;
@@ -1693,7 +1693,7 @@ int run_search(sph_ctx *ctx, sph_particles *parts, int pass)
     SearchArgs a{};
     a.pos4 = ctx->pos4;
     a.h = parts->h;
-    a.active = force ? (ctx->bin_mode ? ctx->bin_active : nullptr) : ctx->active;
+    a.active = force || all ? (ctx->bin_mode ? ctx->bin_active : nullptr) : ctx->active;
     a.boxes = ctx->d_boxes;
     a.cell_start = ctx->cell_start;
     a.cell_reach = ctx->cell_tmp;
@@ -1714,7 +1714,7 @@ int run_search(sph_ctx *ctx, sph_particles *parts, int pass)
     a.cnt = P.cnt;
     a.radius = P.radius;
     a.counters = ctx->counters;
-    const unsigned few = few_rows(ctx);
+    const unsigned few = list_few_rows(ctx);
     if (force) {
         a.run_if = ctx->counters + C_GROWN;
         a.run_above = few;
@@ -1771,7 +1771,7 @@ int run_mark(sph_ctx *ctx, sph_particles *parts)
     m.dirty = P.rows + 3 * cap;
     m.nb = ctx->n_boxes;
     m.grow = ctx->lists.grow;
-    m.run_upto = few_rows(ctx);
+    m.run_upto = list_few_rows(ctx);
     const unsigned blocks = (unsigned)std::min<int64_t>(912, m.run_upto / 8 + 1);
     if (ctx->adaptive) k_mark_dirty<1><<<blocks, 256, 0, ctx->stream>>>(m);
     else k_mark_dirty<0><<<blocks, 256, 0, ctx->stream>>>(m);
