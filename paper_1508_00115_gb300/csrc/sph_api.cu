@@ -396,14 +396,11 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
         if (rc) return rc;
     }
     if (n > 0) {
-        int rc = init_active(ctx);
-        if (rc) return rc;
-        rc = reset_h_brackets(ctx);
+        int rc = density_begin(ctx, ctx->bin_mode);
         if (rc) return rc;
         // passes without lists: every tile at first (and after a rebuild), then those with a
         // target left; individual time-steps: those with a target whose step ends
         bool all_tiles = !ctx->bin_mode, compact = ctx->bin_mode;
-        SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_PREC, 0, sizeof(unsigned long long), ctx->stream));
         if (lists_apply(ctx)) {
             rc = ensure_lists(ctx, 0);
             if (rc) return rc;
@@ -520,11 +517,8 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
                 use_lists = lists_apply(ctx) && settled;
                 fresh = true;
                 again = some_done = partial = false;
-                rc = init_active(ctx);
+                rc = density_begin(ctx, ctx->bin_mode);  // slots were permuted
                 if (rc) return rc;
-                rc = reset_h_brackets(ctx);  // slots were permuted
-                if (rc) return rc;
-                SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_PREC, 0, sizeof(unsigned long long), ctx->stream));
                 all_tiles = !ctx->bin_mode;
                 compact = ctx->bin_mode;
             }
@@ -907,15 +901,10 @@ static int graph_step(sph_ctx *ctx, sph_particles *parts, double dt, int passes)
         rc = sync_h(ctx, parts);
         if (rc) return rc;
     }
-    const int n = (int)ctx->n;
-    SPH_CUDA(ctx, cudaMemsetAsync(ctx->active, 1, n, ctx->stream));
-    rc = reset_h_brackets(ctx);
+    rc = density_begin(ctx, false);
     if (rc) return rc;
-    SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_UNCONV, 0, 2 * sizeof(unsigned long long), ctx->stream));
-    SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_PREC, 0, sizeof(unsigned long long), ctx->stream));
     const bool lists = lists_apply(ctx);
     ctx->lists.grow = kListGrow;
-    SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_LOST, 0, sizeof(unsigned long long), ctx->stream));
     if (lists) {
         rc = lists_begin(ctx, false);
         if (rc) return rc;

@@ -445,7 +445,7 @@ int tree_read_device(sph_ctx *ctx);                             // sph_tree.cu (
 int tree_cell_keys_out(sph_ctx *ctx, int32_t *dev_keys);        // sph_tree.cu
 int tree_shrink_count(sph_ctx *ctx, sph_particles *parts);      // sph_tree.cu
 int tree_leaf_hcur(sph_ctx *ctx, sph_particles *parts);         // sph_tree.cu (before a force pass)
-int reset_h_brackets(sph_ctx *ctx);                             // sph_pairs.cu
+int density_begin(sph_ctx *ctx, bool bins);                      // sph_pairs.cu
 // individual time-steps, sph_integrate.cu
 int bin_permute(sph_ctx *ctx, sph_particles *parts);  // after each permutation: bins, kept state, prediction
 int bin_active(sph_ctx *ctx, unsigned long long *n_active);  // active mask at ctx->bin_now (host read)

@@ -1964,12 +1964,26 @@ int ensure_sym(sph_ctx *ctx)
 }
 
 // Open brackets: lower end 0, upper end kHUnbounded (bytes 0x7f: 3.39e38).
-int reset_h_brackets(sph_ctx *ctx)
+// Start of a density call: its targets (src, or every particle), open brackets of h, and the
+// call's counters (one launch in place of six copies and fills).
+__global__ void k_density_begin(uint8_t *__restrict__ active, const uint8_t *__restrict__ src, float *__restrict__ lo,
+                                float *__restrict__ hi, int n, unsigned long long *__restrict__ c)
 {
-    const int64_t n = ctx->n;
-    if (n <= 0) return SPH_OK;
-    SPH_CUDA(ctx, cudaMemsetAsync(ctx->h_lo, 0, sizeof(float) * n, ctx->stream));
-    SPH_CUDA(ctx, cudaMemsetAsync(ctx->h_hi, 0x7f, sizeof(float) * n, ctx->stream));
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) c[C_UNCONV] = c[C_HFLAG] = c[C_PREC] = c[C_LOST] = 0ull;
+    if (i >= n) return;
+    active[i] = src ? src[i] : (uint8_t)1;
+    lo[i] = 0.f;
+    hi[i] = __uint_as_float(0x7f7f7f7fu);  // above kHUnbounded
+}
+
+// bins: the particles whose step ends now (individual time-steps)
+int density_begin(sph_ctx *ctx, bool bins)
+{
+    const int n = (int)ctx->n;
+    k_density_begin<<<(unsigned)std::max(1, (n + 255) / 256), 256, 0, ctx->stream>>>(
+        ctx->active, bins ? ctx->bin_active : nullptr, ctx->h_lo, ctx->h_hi, n, ctx->counters);
+    SPH_LAUNCH(ctx, "density begin");
     return SPH_OK;
 }
 

@@ -274,3 +274,32 @@ def test_limiter_batched_boxes_match_each_box_alone():
         for k in ("vx", "vy", "vz", "u", "h"):
             x, y = gb[k][sl][ib], g[k][ia]
             assert np.abs(x - y).max() <= 1e-5 * np.abs(y).max(), k
+
+
+def test_limiter_passes_share_a_particle_or_not():
+    """Twelve copies of a blast in one context (more active particles than warps: one warp
+    each) against one copy alone (several warps per particle): the same bins and raises."""
+    from paper_1508_00115_gb300 import binding
+    d = _blast(1200, 41)
+    n, copies = d["x"].size, 12
+    many = {k: np.concatenate([d[k]] * copies) for k in inputs.FIELDS}
+    out = []
+    for field, boxes in ((d, None), (many, [n * k for k in range(copies + 1)])):
+        m = field["x"].size
+        ctx = binding.Context(m, flags=binding.SPH_FLAG_BIN_LIMITER, box_offsets=boxes)
+        parts = binding.Particles(field)
+        ctx.build_cells(parts)
+        ctx.density(parts)
+        ctx.force(parts)
+        g = parts.numpy()
+        dt_max = 16.0 * float(np.min(0.1 * g["h"].astype(np.float64) / g["vsig"].astype(np.float64)))
+        _, st = ctx.step_bins(parts, dt_max, 8)
+        bins = np.empty(m, np.int8)
+        bins[ctx.permutation()] = ctx.bins()
+        out.append((bins, st))
+        ctx.close()
+    (b1, s1), (b2, s2) = out
+    assert s1["limited"] > 0 and s1["woken"] > 0
+    assert np.array_equal(np.tile(b1, copies), b2)
+    for k in ("updates", "limited", "woken"):
+        assert s2[k] == copies * s1[k], k
