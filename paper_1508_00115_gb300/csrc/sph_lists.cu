@@ -26,8 +26,12 @@
 namespace sph {
 
 constexpr int kCodes = 1024;      // hits of a batch written out at once
-constexpr int kListThreads = 256;
-constexpr int kSearchBlocks = 3;  // resident blocks per SM the kernels are compiled for
+constexpr int kListThreads = 128;
+// resident blocks per SM the search is compiled for: more warps where there are tiles for all of
+// them many times over, else more registers for each (ms per call with 5 and with 7: 512 boxes
+// of 37 k 154.3, 151.0; Sedov 2 M 13.5, 13.3; clustered 2 M 19.1, 19.8; clustered 200 k 10.5,
+// 10.9; 32 k uniform 0.475, 0.50)
+constexpr int kSearchFew = 5, kSearchMany = 7;
 // the sums wait for scattered reads: a lane has both names of a step in flight, and five blocks
 // of four warps leave it the registers for that (Sedov 2 M, 19 M in 512 boxes, ms per call: one
 // name after the other at 24 warps per SM 14.4, 160; both at 24 warps 14.7, 154; at 20 13.4,
@@ -341,8 +345,8 @@ __device__ __forceinline__ void emit_batch(const SearchArgs &a, const unsigned (
 }
 
 // MODE: 0 = uniform grid, 1 = adaptive cells
-template <int MODE>
-__global__ void __launch_bounds__(kListThreads, kSearchBlocks) k_search(SearchArgs a)
+template <int MODE, int BLOCKS>
+__global__ void __launch_bounds__(kListThreads, BLOCKS) k_search(SearchArgs a)
 {
     if (a.run_if && *a.run_if <= a.run_above && !(a.or_if && (*a.or_if & 3ull))) return;
     constexpr bool LIST = MODE == 1;
@@ -1675,8 +1679,10 @@ static int search_optin(sph_ctx *ctx)
     static bool done = false;
     if (done) return SPH_OK;
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    SPH_CUDA(ctx, cudaFuncSetAttribute(k_search<0>, at, (int)kSearchSmem));
-    SPH_CUDA(ctx, cudaFuncSetAttribute(k_search<1>, at, (int)kSearchSmem));
+    SPH_CUDA(ctx, cudaFuncSetAttribute(k_search<0, kSearchFew>, at, (int)kSearchSmem));
+    SPH_CUDA(ctx, cudaFuncSetAttribute(k_search<0, kSearchMany>, at, (int)kSearchSmem));
+    SPH_CUDA(ctx, cudaFuncSetAttribute(k_search<1, kSearchFew>, at, (int)kSearchSmem));
+    SPH_CUDA(ctx, cudaFuncSetAttribute(k_search<1, kSearchMany>, at, (int)kSearchSmem));
     done = true;
     return SPH_OK;
 }
@@ -1729,11 +1735,14 @@ int run_search(sph_ctx *ctx, sph_particles *parts, int pass, bool all)
     a.grow = force ? 1.f : ctx->lists.grow;
     a.wbits = name_bits(ctx);
     a.force = force ? 1 : 0;
-    const int g = list_grid(ctx, kListThreads, kSearchBlocks);
+    const bool many = ctx->n >= (ctx->adaptive ? 8000000 : 1000000);
+    const int g = list_grid(ctx, kListThreads, many ? kSearchMany : kSearchFew);
     cudaEvent_t end = nullptr;
     timer_begin(ctx, force ? 1 : 0, &end);
-    if (ctx->adaptive) k_search<1><<<g, kListThreads, kSearchSmem, ctx->stream>>>(a);
-    else k_search<0><<<g, kListThreads, kSearchSmem, ctx->stream>>>(a);
+    if (ctx->adaptive && many) k_search<1, kSearchMany><<<g, kListThreads, kSearchSmem, ctx->stream>>>(a);
+    else if (ctx->adaptive) k_search<1, kSearchFew><<<g, kListThreads, kSearchSmem, ctx->stream>>>(a);
+    else if (many) k_search<0, kSearchMany><<<g, kListThreads, kSearchSmem, ctx->stream>>>(a);
+    else k_search<0, kSearchFew><<<g, kListThreads, kSearchSmem, ctx->stream>>>(a);
     timer_end(ctx, end);
     SPH_LAUNCH(ctx, "neighbour search");
     if (pass == 0) return SPH_OK;
