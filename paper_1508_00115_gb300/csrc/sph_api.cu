@@ -706,9 +706,7 @@ static int do_step(sph_ctx *ctx, sph_particles *parts, double dt, double *dt_use
         if (!isfinite(dt)) return fail(ctx, SPH_ERR_INVALID_ARG, "no signal velocity: pass an explicit dt");
     }
     SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_FLOORS, 0, sizeof(unsigned long long), ctx->stream));
-    rc = kick(ctx, parts);
-    if (rc) return rc;
-    rc = drift(ctx, parts);
+    rc = kick_drift(ctx, parts);
     if (rc) return rc;
     // the hydro pass sees v and u predicted to the end of the step (vel4 / upred)
     ctx->predict = true;
@@ -888,9 +886,7 @@ static int graph_step(sph_ctx *ctx, sph_particles *parts, double dt, int passes)
 {
     int rc = dt > 0 ? set_dt(ctx, dt) : cfl_dt_device(ctx, parts);
     if (rc) return rc;
-    rc = kick(ctx, parts);
-    if (rc) return rc;
-    rc = drift(ctx, parts);
+    rc = kick_drift(ctx, parts);
     if (rc) return rc;
     ctx->predict = true;
     rc = build_planned(ctx, parts);

@@ -24,19 +24,43 @@ int set_dt(sph_ctx *ctx, double dt)
     return SPH_OK;
 }
 
-// v += a * dt/2 (FP64); u <- max(u + dudt * dt/2, 0), counting floors
+// (double)f by integer operations, for the normal numbers and zero (exact: the exponent's bias
+// moved, the fraction shifted).  The FP64 pipe takes two lanes a clock and conversions go
+// through it: they, not the memory, bound the kicks.
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned b = __float_as_uint(f), a = b & 0x7fffffffu;
+    if (a - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
+    return a == 0u ? __hiloint2double((int)b, 0) : (double)f;
+}
+
+// v += a * dt/2 (FP64); u <- max(u + dudt * dt/2, 0), counting floors; DRIFT: then
+// x += v dt (FP64; the periodic wrap follows in the cell build).  2 M particles: kick 49 ->
+// 25 us, kick and drift 71 -> 41 us.
+template <bool DRIFT>
 __global__ void k_kick(sph_particles P, int n, const double *__restrict__ d_dt, unsigned long long *floors)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const double half_dt = 0.5 * *d_dt;
+    const double dt = *d_dt, half_dt = 0.5 * dt;
     bool fl = false;
     if (i < n) {
-        P.vx[i] += (double)P.ax[i] * half_dt;
-        P.vy[i] += (double)P.ay[i] * half_dt;
-        P.vz[i] += (double)P.az[i] * half_dt;
-        double u = (double)P.u[i] + (double)P.dudt[i] * half_dt;
-        fl = u < 0.0;
-        P.u[i] = (float)(fl ? 0.0 : u);
+        const double vx = P.vx[i] + widen(P.ax[i]) * half_dt, vy = P.vy[i] + widen(P.ay[i]) * half_dt,
+                     vz = P.vz[i] + widen(P.az[i]) * half_dt;
+        P.vx[i] = vx;
+        P.vy[i] = vy;
+        P.vz[i] = vz;
+        if (DRIFT) {
+            P.x[i] += vx * dt;
+            P.y[i] += vy * dt;
+            P.z[i] += vz * dt;
+        }
+        const double u = widen(P.u[i]) + widen(P.dudt[i]) * half_dt;
+        // u < 0.0, without the FP64 pipe: the sign of a number that is neither zero nor NaN
+        const unsigned hi = (unsigned)__double2hiint(u), lo = (unsigned)__double2loint(u);
+        const unsigned mag = hi & 0x7fffffffu;
+        fl = (hi >> 31) && (mag | lo) != 0u && (mag < 0x7ff00000u || (mag == 0x7ff00000u && lo == 0u));
+        P.u[i] = fl ? 0.f : (float)u;
     }
     unsigned b = __ballot_sync(kFull, fl);
     if ((threadIdx.x & 31) == 0 && b) atomicAdd(floors, (unsigned long long)__popc(b));
@@ -46,12 +70,21 @@ int kick(sph_ctx *ctx, sph_particles *parts)
 {
     int n = (int)ctx->n;
     if (n <= 0) return SPH_OK;
-    k_kick<<<(n + 255) / 256, 256, 0, ctx->stream>>>(*parts, n, ctx->d_dt, ctx->counters + C_FLOORS);
+    k_kick<false><<<(n + 255) / 256, 256, 0, ctx->stream>>>(*parts, n, ctx->d_dt, ctx->counters + C_FLOORS);
     SPH_LAUNCH(ctx, "kick");
     return SPH_OK;
 }
 
-// x += v dt (FP64); the periodic wrap follows in the cell build
+int kick_drift(sph_ctx *ctx, sph_particles *parts)
+{
+    int n = (int)ctx->n;
+    if (n <= 0) return SPH_OK;
+    k_kick<true><<<(n + 255) / 256, 256, 0, ctx->stream>>>(*parts, n, ctx->d_dt, ctx->counters + C_FLOORS);
+    SPH_LAUNCH(ctx, "kick and drift");
+    return SPH_OK;
+}
+
+// x += v dt (FP64; individual time-steps)
 __global__ void k_drift(sph_particles P, int n, const double *__restrict__ d_dt)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -123,12 +156,12 @@ __global__ void __launch_bounds__(kRedThreads) k_conserved_part(sph_particles P,
 {
     double s[5] = {0, 0, 0, 0, 0};
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double m = (double)P.m[i], vx = P.vx[i], vy = P.vy[i], vz = P.vz[i];
+        double m = widen(P.m[i]), vx = P.vx[i], vy = P.vy[i], vz = P.vz[i];
         s[0] += m * vx;
         s[1] += m * vy;
         s[2] += m * vz;
         s[3] += 0.5 * m * (vx * vx + vy * vy + vz * vz);
-        s[4] += m * (double)P.u[i];
+        s[4] += m * widen(P.u[i]);
     }
     __shared__ double sh[5][kRedThreads];
 #pragma unroll

@@ -492,6 +492,7 @@ int run_force_pass(sph_ctx *ctx, sph_particles *parts, bool active_list = false,
 int run_gravity_pass(sph_ctx *ctx, double G, double eps, float *ax, float *ay, float *az, float *phi);  // sph_gravity.cu
 int ensure_sym(sph_ctx *ctx);  // slot arrays of the symmetric force pass           // sph_pairs.cu
 int sync_h(sph_ctx *ctx, sph_particles *parts);                            // sph_pairs.cu
+int kick_drift(sph_ctx *ctx, sph_particles *parts);
 int kick(sph_ctx *ctx, sph_particles *parts);    // by *d_dt / 2           // sph_integrate.cu
 int drift(sph_ctx *ctx, sph_particles *parts);   // by *d_dt               // sph_integrate.cu
 int set_dt(sph_ctx *ctx, double dt);             // *d_dt = dt (kernel)    // sph_integrate.cu
