@@ -3,6 +3,10 @@
 //            the velocity divergence/curl, and the per-particle quantities needed
 //            before the pressure gradient (EOS, grad-h factor, Balsara switch);
 //   force:   Eq. 2 in the Gadget-2 form with signal-velocity viscosity.
+// Here without neighbour lists: every pass searches for itself.  sph_lists.cu runs both over
+// lists instead, wherever its lists apply; these kernels run where they do not (the axis
+// sweep, uniform grids beyond 2^25 slots, adaptive cells before a density call has
+// converged, lists that found no room), and the symmetric force pass always.
 //
 // Work decomposition (replaces the paper's self/pair tasks and task scheduler):
 // a tile is up to TW (16 or 32) target particles of one cell, one lane per
