@@ -1568,8 +1568,9 @@ void free_lists(sph_ctx *ctx)
     P = ListPool();
 }
 
-// Arrays for the lists (never inside a capture): `pages` of them at least.  Where the
-// device has no room the lists are switched off and the kernels of sph_pairs.cu run.
+// Arrays for the lists (never inside a capture): `pages` of them at least.  Where they would
+// take more than half of the device's free memory, which other allocations of the call may
+// need, the lists are switched off and the kernels of sph_pairs.cu run.
 int ensure_lists(sph_ctx *ctx, int64_t pages)
 {
     ListPool &P = ctx->lists;
@@ -1583,7 +1584,13 @@ int ensure_lists(sph_ctx *ctx, int64_t pages)
         return false;
     };
     bool ok = true;
-    if (P.cap < cap) {
+    if (P.cap < cap || P.cap_pages < pages) {
+        const size_t need = (P.cap < cap ? 29 * (size_t)cap : 0) +
+                            (P.cap_pages < pages ? 4 * (kPage + 1) * (size_t)pages : 0);
+        size_t left = 0, total = 0;
+        ok = cudaMemGetInfo(&left, &total) == cudaSuccess && need <= left / 2;
+    }
+    if (ok && P.cap < cap) {
         ok = room(&P.head, sizeof(int) * cap) && room(&P.cnt, sizeof(int) * cap) &&
              room(&P.radius, sizeof(float) * cap) && room(&P.rows, 4 * sizeof(int) * cap) &&
              room(&P.mark, ((size_t)cap + 3) / 4 * 4) &&
