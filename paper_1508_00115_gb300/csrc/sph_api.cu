@@ -396,15 +396,13 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
         if (rc) return rc;
     }
     if (n > 0) {
-        int rc = density_begin(ctx, ctx->bin_mode);
+        int rc = lists_apply(ctx) ? ensure_lists(ctx, 0) : SPH_OK;
+        if (rc) return rc;
+        rc = density_begin(ctx, ctx->bin_mode);
         if (rc) return rc;
         // passes without lists: every tile at first (and after a rebuild), then those with a
         // target left; individual time-steps: those with a target whose step ends
         bool all_tiles = !ctx->bin_mode, compact = ctx->bin_mode;
-        if (lists_apply(ctx)) {
-            rc = ensure_lists(ctx, 0);
-            if (rc) return rc;
-        }
         ctx->lists.ready = false;
         // adaptive cells take any guess of h, and one off by decades asks for lists of 100,000
         // names, walked by every Newton step: until a call has converged, passes without lists
@@ -524,7 +522,7 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
             }
         }
         unconv += lost;
-        if (use_lists && !partial && ctx->h_counters[C_GROWN]) {
+        if (use_lists && !partial && !ctx->sym_force && ctx->h_counters[C_GROWN]) {
             rc = run_mark(ctx, parts);
             if (rc) return rc;
         }
@@ -926,7 +924,7 @@ static int graph_step(sph_ctx *ctx, sph_particles *parts, double dt, int passes)
     }
     k_step_flags<<<1, 1, 0, ctx->stream>>>(ctx->counters);
     SPH_LAUNCH(ctx, "step flags");
-    if (lists) {
+    if (lists && !ctx->sym_force) {
         rc = run_mark(ctx, parts);
         if (rc) return rc;
     }

@@ -201,7 +201,7 @@ struct ListPool {
     int *head = nullptr, *cnt = nullptr;  // per slot: first page, names
     float *radius = nullptr;    // per slot: list radius
     int *rows = nullptr;        // 4 x cap: targets left by the last two passes, grown, dirty
-    uint8_t *mark = nullptr;    // dirty targets (zero between the force passes)
+    uint8_t *mark = nullptr;    // dirty targets of the present density call
     int64_t cap = 0, cap_pages = 0;
     bool off = false;           // no room on the device
     bool ready = false;         // lists of the current cells, from the last density call

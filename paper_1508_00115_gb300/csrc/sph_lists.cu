@@ -603,7 +603,6 @@ struct SearchOneArgs {
     const int *__restrict__ leaf_of;      // adaptive cells
     unsigned run_upto;                    // run only up to so many rows
     const unsigned long long *unless;     // ... and only if this is zero
-    uint8_t *mark;                        // marks of the rows, to be cleared (null: none)
 };
 
 template <int MODE>
@@ -611,9 +610,6 @@ __global__ void __launch_bounds__(256) k_search_one(SearchOneArgs b)
 {
     const SearchArgs &a = b.s;
     const unsigned long long nr = *b.n_rows;
-    if (b.mark)
-        for (unsigned long long u = blockIdx.x * blockDim.x + threadIdx.x; u < nr; u += gridDim.x * blockDim.x)
-            b.mark[b.rows[u]] = 0;
     if (nr == 0ull || nr > b.run_upto || (*b.unless & 3ull)) return;
     constexpr bool LIST = MODE == 1;
     const int lane = threadIdx.x & 31;
@@ -1291,7 +1287,7 @@ __global__ void __launch_bounds__(kSumThreads, kSumBlocks) k_density_l(DensityLi
 
 // The targets that the lists of a few grown particles' neighbours miss: for every j whose h
 // outgrew the radius its neighbours searched with, the targets of its own list (searched at
-// the new h) beyond that radius, each once (mark: zero, and zero again after the search).
+// the new h) beyond that radius, each once (mark: zero from the start of the density call).
 // pos4.w still holds the h that the searches used; h the converged one.
 struct MarkArgs {
     SumArgs s;
@@ -1593,8 +1589,7 @@ int ensure_lists(sph_ctx *ctx, int64_t pages)
     if (ok && P.cap < cap) {
         ok = room(&P.head, sizeof(int) * cap) && room(&P.cnt, sizeof(int) * cap) &&
              room(&P.radius, sizeof(float) * cap) && room(&P.rows, 4 * sizeof(int) * cap) &&
-             room(&P.mark, ((size_t)cap + 3) / 4 * 4) &&
-             cudaMemsetAsync(P.mark, 0, ((size_t)cap + 3) / 4 * 4, ctx->stream) == cudaSuccess;
+             room(&P.mark, ((size_t)cap + 3) / 4 * 4);
         P.cap = cap;
     }
     if (ok && P.cap_pages < pages) {
@@ -1764,7 +1759,6 @@ int run_search(sph_ctx *ctx, sph_particles *parts, int pass, bool all)
     b.unless = ctx->counters + C_STALE;
     b.keys = ctx->keys;
     b.leaf_of = ctx->tree.leaf_of;
-    b.mark = force ? P.mark : nullptr;
     if (ctx->adaptive) k_search_one<1><<<blocks, 256, 0, ctx->stream>>>(b);
     else k_search_one<0><<<blocks, 256, 0, ctx->stream>>>(b);
     SPH_LAUNCH(ctx, "search of single targets");

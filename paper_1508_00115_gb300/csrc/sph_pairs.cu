@@ -1967,11 +1967,12 @@ int ensure_sym(sph_ctx *ctx)
     return SPH_OK;
 }
 
-// Open brackets: lower end 0, upper end kHUnbounded (bytes 0x7f: 3.39e38).
-// Start of a density call: its targets (src, or every particle), open brackets of h, and the
-// call's counters (one launch in place of six copies and fills).
+// Start of a density call: its targets (src, or every particle), open brackets of h, no target
+// marked for the force pass's search (mark; a call's marks may never meet one), and the call's
+// counters (one launch in place of six copies and fills).
 __global__ void k_density_begin(uint8_t *__restrict__ active, const uint8_t *__restrict__ src, float *__restrict__ lo,
-                                float *__restrict__ hi, int n, unsigned long long *__restrict__ c)
+                                float *__restrict__ hi, uint8_t *__restrict__ mark, int n,
+                                unsigned long long *__restrict__ c)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) c[C_UNCONV] = c[C_HFLAG] = c[C_PREC] = c[C_LOST] = 0ull;
@@ -1979,14 +1980,16 @@ __global__ void k_density_begin(uint8_t *__restrict__ active, const uint8_t *__r
     active[i] = src ? src[i] : (uint8_t)1;
     lo[i] = 0.f;
     hi[i] = __uint_as_float(0x7f7f7f7fu);  // above kHUnbounded
+    if (mark) mark[i] = 0;
 }
 
 // bins: the particles whose step ends now (individual time-steps)
 int density_begin(sph_ctx *ctx, bool bins)
 {
     const int n = (int)ctx->n;
+    uint8_t *mark = lists_apply(ctx) ? ctx->lists.mark : nullptr;
     k_density_begin<<<(unsigned)std::max(1, (n + 255) / 256), 256, 0, ctx->stream>>>(
-        ctx->active, bins ? ctx->bin_active : nullptr, ctx->h_lo, ctx->h_hi, n, ctx->counters);
+        ctx->active, bins ? ctx->bin_active : nullptr, ctx->h_lo, ctx->h_hi, mark, n, ctx->counters);
     SPH_LAUNCH(ctx, "density begin");
     return SPH_OK;
 }

@@ -102,3 +102,32 @@ def test_leaf_too_large_for_its_names():
     s = oracle_state(g)
     check_density(g, s)
     check_force(g, s)
+
+
+def _lowered(parts, share, factor, seed):
+    pick = torch.as_tensor(np.random.default_rng(seed).random(parts.t["h"].numel()) < share, device="cuda")
+    parts.t["h"][pick] *= factor
+
+
+@pytest.mark.parametrize("flag", ["uniform", "adaptive", "autotune"])
+def test_density_calls_that_no_force_follows(flag):
+    """The targets a density call marks for the force pass's search are that call's alone: calls
+    without a force pass after them (and the tuner's own) leave nothing to the next."""
+    from paper_1508_00115_gb300 import binding
+    flags = {"uniform": 0, "adaptive": binding.SPH_FLAG_ADAPTIVE, "autotune": binding.SPH_FLAG_AUTOTUNE}[flag]
+    d = inputs.plummer_mix(6000, seed=61, n_halos=6) if flag == "adaptive" else inputs.uniform(6000, seed=62)
+    d = inputs.random_velocities(d, 0.3, 63)
+    ctx = binding.Context(6000, flags=flags | binding.SPH_FLAG_NGB_HASH, cell_factor=1.5)
+    parts = binding.Particles(d)
+    for k in range(5):
+        ctx.build_cells(parts)
+        ctx.density(parts)
+        _lowered(parts, 0.01, 0.9, 64 + k)
+    ctx.build_cells(parts)
+    ctx.density(parts)
+    ctx.force(parts)
+    g = parts.numpy()
+    g["perm"], g["ngb_hash"] = ctx.permutation(), ctx.ngb_hash()
+    s = oracle_state(g)
+    check_density(g, s)
+    check_force(g, s)
