@@ -1325,6 +1325,7 @@ __global__ void __launch_bounds__(256) k_mark_dirty(MarkArgs a)
         const uint32_t e0 = LIST ? a.s.list_off[leaf] : 0u;
         const float4 pi = a.s.pos4[i];
         const float hf = a.h[i];
+        const float reach = LIST ? pi.w * a.grow : fminf(pi.w * a.grow, 2.f * L * (1.f - 1e-6f));
         const float top = fmaf(hf, hf, 2.f * kBandK * hf * (hf + L));
         walk_list<32>(a.s, a.s.cnt[i], a.s.head[i], lane, [&](Two name, TwoBool ok) {
 #pragma unroll
@@ -1335,7 +1336,9 @@ __global__ void __launch_bounds__(256) k_mark_dirty(MarkArgs a)
                 const float4 pj = a.s.pos4[j];
                 const float dx = pi.x - (pj.x + sx), dy = pi.y - (pj.y + sy), dz = pi.z - (pj.z + sz);
                 const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                const float held = fmaxf(pi.w, pj.w) * a.grow * (1.f - 1e-5f);
+                // what j's list holds: pairs within j's own list radius (on adaptive cells as far as
+                // its leaf's entries reach, which may end below h_j's growth) or i's reach
+                const float held = fmaxf(reach, __ldg(a.s.radius + j)) * (1.f - 1e-5f);
                 if (j != i && r2 < top && r2 > held * held && (a.mask == nullptr || a.mask[j])) {
                     // (one writer wins: bytes are marked through their word)
                     const unsigned bit = 1u << (8 * (j & 3));

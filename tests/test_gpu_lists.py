@@ -131,3 +131,42 @@ def test_density_calls_that_no_force_follows(flag):
     s = oracle_state(g)
     check_density(g, s)
     check_force(g, s)
+
+
+def test_source_that_grows_past_a_capped_list_radius():
+    """Adaptive cells: a list ends at 1.15 of the leaf's largest h at the build, here below 1.04 of
+    the (predicted) h that the search took for the source's reach.  Particles that grow from
+    0.92 of theirs into that gap are missed by the neighbour's list, and its force sum has to get
+    them: the pairs of the force pass against all pairs in FP64."""
+    from paper_1508_00115_gb300 import binding
+    n = 20000
+    d = inputs.random_velocities(inputs.uniform(n, seed=71), 0.1, 72)
+    at = np.linspace(0.0, 1.0, 4097)  # density exp(2 cos 2 pi x): h changes by a third within h
+    mass = np.cumsum(np.exp(2.0 * np.cos(2.0 * np.pi * at)))
+    d["x"] = np.interp(d["x"], (mass - mass[0]) / (mass[-1] - mass[0]), at)
+    ctx = binding.Context(n, flags=binding.SPH_FLAG_ADAPTIVE | binding.SPH_FLAG_HPREDICT, cell_factor=1.25,
+                          leaf_max=32, h_tol=1e-5)
+    f = np.zeros(binding.SPH_HP_NF32, np.float32)
+    f[135:141] = 1.0
+    f[141] = np.log(1.149)  # every h is predicted to grow by that
+    f[142] = 1.0
+    ctx.hp_load(np.zeros(binding.SPH_HP_NBF16, np.uint16), f)
+    parts = binding.Particles(d)
+    kept = 0
+    for k in range(8):
+        ctx.build_cells(parts)
+        ctx.density(parts)
+        ctx.force(parts)
+        _lowered(parts, 0.003, 0.8, 73 + k)
+        ctx.reset_stats()
+        ctx.step(parts, 1e-9)
+        st = ctx.stats()
+        kept += st["rebuilds"] == 0  # (a rebuild starts from the grown h)
+        x = torch.stack([parts.t[c] for c in ("x", "y", "z")], dim=1)
+        h, pairs = parts.t["h"].double(), 0
+        for i in range(0, n, 2000):
+            dx = x[i:i + 2000, None] - x[None]
+            r2 = ((dx - torch.round(dx)) ** 2).sum(dim=2)
+            pairs += int((r2 < torch.maximum(h[i:i + 2000, None], h[None]) ** 2).sum())
+        assert st["force_pairs"] == pairs - n, k
+    assert kept >= 3
