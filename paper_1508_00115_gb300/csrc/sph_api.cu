@@ -831,6 +831,9 @@ static int do_step_bins(sph_ctx *ctx, sph_particles *parts, double dt_max, int l
     };
     rc = body();
     ctx->bin_mode = false;
+    // the lists at hand are those of the last step end's targets; the others' (after an error
+    // there are some) come from earlier builds and name what the cells no longer hold
+    ctx->lists.ready = false;
     if (rc) return rc;
     ctx->hydro_valid = true;  // all particles were active at dt_max
     if (bs) {
@@ -1516,6 +1519,15 @@ const char *sph_last_error(const sph_ctx *ctx)
 {
     if (!ctx) return "null context";
     return ctx->err.c_str();
+}
+
+// For the tests, not declared in sph.h: let something of the context run out early, to reach
+// the calls' behaviour there.  which 0: the limiter's passes from now on.  value < 0: no limit.
+int sph_test_limit(sph_ctx *ctx, int32_t which, int64_t value)
+{
+    if (!ctx || which != 0) return SPH_ERR_INVALID_ARG;
+    ctx->limits.limiter_passes = value;
+    return SPH_OK;
 }
 
 void sph_destroy(sph_ctx *ctx)

@@ -733,7 +733,9 @@ int bin_limit(sph_ctx *ctx, sph_particles *parts, bool all, int64_t *sweeps)
     // raises is at most SPH_MAX_BINS / K + 1 long; passes beyond that find nothing
     const int max_sweeps = SPH_MAX_BINS + 2;
     for (int k = 0;; ++k) {
-        if (k >= max_sweeps) return fail(ctx, SPH_ERR_TIMEOUT, "time-step limiter did not settle");
+        if (k >= max_sweeps || ctx->limits.limiter_passes == 0)
+            return fail(ctx, SPH_ERR_TIMEOUT, "time-step limiter did not settle");
+        if (ctx->limits.limiter_passes > 0) --ctx->limits.limiter_passes;
         k_lim_reset<<<(unsigned)((nc + 255) / 256), 256, 0, ctx->stream>>>(
             ctx->lim_cmax, ctx->lim_cmax + nc, dirty[(k + 1) & 1], nc, ctx->counters, k == 0 ? 1 : 0);
         SPH_LAUNCH(ctx, "limiter reset");

@@ -367,6 +367,11 @@ struct sph_ctx {
 
     sph::ListPool lists;  // neighbour lists
 
+    // what runs out where the tests want it to (sph_test_limit); below 0: no limit
+    struct {
+        int64_t limiter_passes = -1;  // limiter passes left
+    } limits;
+
     // statistics
     sph_stats st{};
     std::vector<sph::Timer> timers;

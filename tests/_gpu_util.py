@@ -1,5 +1,7 @@
 """Shared helpers of the GPU parity tests: run the CUDA path through the C-ABI and
 rebuild, from its outputs, the oracle state in the same (cell) order."""
+import ctypes
+
 import numpy as np
 
 import oracle
@@ -22,6 +24,24 @@ def gpu_hydro(d: dict, **params):
         out["ngb_hash"] = ctx.ngb_hash()
     out["stats"] = ctx.stats()
     return ctx, parts, out
+
+
+def set_limit(ctx, which: int, value: int):
+    """sph_test_limit: let something of the context run out early (-1: as it comes)."""
+    from paper_1508_00115_gb300 import binding
+    assert binding.lib().sph_test_limit(ctx.h, ctypes.c_int32(which), ctypes.c_int64(value)) == binding.SPH_OK
+
+
+def force_pairs(parts) -> int:
+    """Directed pairs r_ij < max(h_i, h_j), j != i, of the particles in a box of side 1 (FP64)."""
+    import torch
+    x = torch.stack([parts.t[c] for c in ("x", "y", "z")], dim=1)
+    h, n, pairs = parts.t["h"].double(), x.shape[0], 0
+    for i in range(0, n, 2000):
+        dx = x[i:i + 2000, None] - x[None]
+        r2 = ((dx - torch.round(dx)) ** 2).sum(dim=2)
+        pairs += int((r2 < torch.maximum(h[i:i + 2000, None], h[None]) ** 2).sum())
+    return pairs - n
 
 
 def oracle_state(g: dict, box: float = 1.0) -> oracle.State:

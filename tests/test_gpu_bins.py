@@ -303,3 +303,29 @@ def test_limiter_passes_share_a_particle_or_not():
     assert np.array_equal(np.tile(b1, copies), b2)
     for k in ("updates", "limited", "woken"):
         assert s2[k] == copies * s1[k], k
+
+
+@pytest.mark.parametrize("adaptive", [False, True])
+def test_force_after_bins_that_ended_early(adaptive):
+    """sph_step_bins that fails after some step ends (the limiter's passes run out) leaves lists of
+    the last step end's targets only: a force pass called there sums over all pairs again."""
+    from paper_1508_00115_gb300 import binding
+    from _gpu_util import force_pairs, set_limit
+    flags = binding.SPH_FLAG_BIN_LIMITER | (binding.SPH_FLAG_ADAPTIVE if adaptive else 0)
+    d = _blast(1200, 41)
+    ctx, parts = _hydro_ctx(d, flags=flags)
+    g = parts.numpy()
+    dt_max = 16.0 * 0.1 * float(np.min(g["h"].astype(np.float64) / g["vsig"].astype(np.float64)))
+    _, st = ctx.step_bins(parts, dt_max, 8)
+    assert st["substeps"] > 4 and st["limit_sweeps"] > 8
+    for share in (0.5, 0.8):
+        ctx, parts = _hydro_ctx(d, flags=flags)
+        set_limit(ctx, 0, int(share * st["limit_sweeps"]))
+        with pytest.raises(binding.SphError) as e:
+            ctx.step_bins(parts, dt_max, 8)
+        assert e.value.code == binding.SPH_ERR_TIMEOUT
+        ctx.reset_stats()
+        ctx.force(parts)
+        assert ctx.stats()["force_pairs"] == force_pairs(parts)
+        set_limit(ctx, 0, -1)
+        ctx.step(parts, 0.1 * dt_max / 16.0)

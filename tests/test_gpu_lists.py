@@ -8,7 +8,7 @@ import pytest
 
 from paper_1508_00115_gb300 import inputs
 
-from _gpu_util import check_density, check_force, oracle_state
+from _gpu_util import check_density, check_force, force_pairs, oracle_state
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -162,11 +162,5 @@ def test_source_that_grows_past_a_capped_list_radius():
         ctx.step(parts, 1e-9)
         st = ctx.stats()
         kept += st["rebuilds"] == 0  # (a rebuild starts from the grown h)
-        x = torch.stack([parts.t[c] for c in ("x", "y", "z")], dim=1)
-        h, pairs = parts.t["h"].double(), 0
-        for i in range(0, n, 2000):
-            dx = x[i:i + 2000, None] - x[None]
-            r2 = ((dx - torch.round(dx)) ** 2).sum(dim=2)
-            pairs += int((r2 < torch.maximum(h[i:i + 2000, None], h[None]) ** 2).sum())
-        assert st["force_pairs"] == pairs - n, k
+        assert st["force_pairs"] == force_pairs(parts), k
     assert kept >= 3
