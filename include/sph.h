@@ -15,10 +15,11 @@
  *   - Every pointer inside sph_particles is a DEVICE pointer owned by the caller
  *     (except for sph_step_host, which takes HOST pointers).  The library never
  *     frees caller memory.  Arrays are structure-of-arrays, length n, contiguous.
- *   - The library owns its scratch (cell arrays, sort buffers, packed FP32
- *     copies, neighbour lists: about 700 B per particle, less where the device has
- *     no room); it allocates it in sph_init / on first use and frees it in
- *     sph_destroy.
+ *   - The library owns its scratch (cell arrays, sort buffers, packed FP32 copies:
+ *     about 190 B per particle; neighbour lists: about 700 B more to start with, up
+ *     to 2.1 KB where lists are long, in no more than half of the memory that is free
+ *     -- without room for them the sums run without lists); it allocates it in
+ *     sph_init / on first use and frees it in sph_destroy.
  *   - Every call enqueues its work on the stream given to sph_init and returns
  *     after the last launch, EXCEPT where a call documents a host read (the
  *     cell-grid size in sph_build_cells, the convergence count in sph_density,

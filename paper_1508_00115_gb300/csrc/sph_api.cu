@@ -396,9 +396,8 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
         if (rc) return rc;
     }
     if (n > 0) {
-        int rc = lists_apply(ctx) ? ensure_lists(ctx, 0) : SPH_OK;
-        if (rc) return rc;
-        rc = density_begin(ctx, ctx->bin_mode);
+        if (lists_fit(ctx)) ensure_lists(ctx, 0);
+        int rc = density_begin(ctx, ctx->bin_mode);
         if (rc) return rc;
         // passes without lists: every tile at first (and after a rebuild), then those with a
         // target left; individual time-steps: those with a target whose step ends
@@ -462,15 +461,12 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
                 if (ctx->h_counters[C_STALE] & 1ull) {
                     // no page left (the sums did not run): a larger pool, or, where the lists
                     // would be far too long, passes without them
-                    const int64_t most = std::min<int64_t>(16 * std::max<int64_t>(ctx->cap, 64), kMaxPages);
-                    const int64_t had = ctx->lists.cap_pages;
-                    if ((ctx->h_counters[C_STALE] & 4ull) || had >= most) {
+                    const int64_t most = lists_most_pages(ctx), had = ctx->lists.cap_pages;
+                    if ((ctx->h_counters[C_STALE] & 4ull) || had >= most ||
+                        !ensure_lists(ctx, std::min(most, 2 * had))) {
                         use_lists = false;
                     } else {
                         again = some_done;  // (those that are done keep a list for the force pass)
-                        rc = ensure_lists(ctx, std::min(most, 2 * had));
-                        if (rc) return rc;
-                        use_lists = lists_apply(ctx);
                         fresh = true;
                     }
                     continue;
@@ -1002,13 +998,13 @@ static int do_steps(sph_ctx *ctx, sph_particles *parts, int n_steps, double dt, 
         rc = tree_prepare_device(ctx, &tree_sig);
         if (rc) return rc;
     }
-    if (lists_apply(ctx)) {  // the pages the last searches took, and half as many again at least
+    if (lists_fit(ctx)) {  // the pages the last searches took, and half as many again where there is room
         rc = read_counters(ctx);
         if (rc) return rc;
         const int64_t used = (int64_t)ctx->h_counters[C_PAGES];
-        if (used + used / 2 > ctx->lists.cap_pages) ctx->lists.ready = false;
-        rc = ensure_lists(ctx, used + used / 2 > ctx->lists.cap_pages ? 2 * used : 0);
-        if (rc) return rc;
+        const bool more = used + used / 2 > ctx->lists.cap_pages;
+        if (more) ctx->lists.ready = false;
+        ensure_lists(ctx, more ? 2 * used : 0);
     }
     // capture one step on a private stream (the caller's may be the legacy default
     // stream, which cannot be captured); the graph is then launched on the caller's
@@ -1522,11 +1518,12 @@ const char *sph_last_error(const sph_ctx *ctx)
 }
 
 // For the tests, not declared in sph.h: let something of the context run out early, to reach
-// the calls' behaviour there.  which 0: the limiter's passes from now on.  value < 0: no limit.
+// the calls' behaviour there.  which 0: the limiter's passes from now on; 1: the free device
+// memory (bytes) that the neighbour lists see.  value < 0: as it comes.
 int sph_test_limit(sph_ctx *ctx, int32_t which, int64_t value)
 {
-    if (!ctx || which != 0) return SPH_ERR_INVALID_ARG;
-    ctx->limits.limiter_passes = value;
+    if (!ctx || which < 0 || which > 1) return SPH_ERR_INVALID_ARG;
+    (which == 0 ? ctx->limits.limiter_passes : ctx->limits.free_bytes) = value;
     return SPH_OK;
 }
 

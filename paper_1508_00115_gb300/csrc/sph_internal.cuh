@@ -203,7 +203,6 @@ struct ListPool {
     int *rows = nullptr;        // 4 x cap: targets left by the last two passes, grown, dirty
     uint8_t *mark = nullptr;    // dirty targets of the present density call
     int64_t cap = 0, cap_pages = 0;
-    bool off = false;           // no room on the device
     bool ready = false;         // lists of the current cells, from the last density call
     bool stale = false;         // ... that do not serve the force pass
     bool settled = false;       // the last density call converged
@@ -370,6 +369,7 @@ struct sph_ctx {
     // what runs out where the tests want it to (sph_test_limit); below 0: no limit
     struct {
         int64_t limiter_passes = -1;  // limiter passes left
+        int64_t free_bytes = -1;      // device memory that is free for the lists
     } limits;
 
     // statistics
@@ -480,8 +480,10 @@ int cell_keys_out(sph_ctx *ctx, int32_t *dev_keys);             // sph_cells.cu
 int run_density_pass(sph_ctx *ctx, sph_particles *parts, bool last_pass, bool active_list,
                      bool if_no_lists = false);                            // sph_pairs.cu
 // sums over neighbour lists, sph_lists.cu
+bool lists_fit(const sph_ctx *ctx);
 bool lists_apply(const sph_ctx *ctx);
-int ensure_lists(sph_ctx *ctx, int64_t pages);  // (outside captures)
+int64_t lists_most_pages(const sph_ctx *ctx);
+bool ensure_lists(sph_ctx *ctx, int64_t pages);  // (outside captures)
 void free_lists(sph_ctx *ctx);
 int lists_begin(sph_ctx *ctx, bool force);
 unsigned list_few_rows(const sph_ctx *ctx);

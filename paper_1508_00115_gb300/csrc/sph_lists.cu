@@ -1545,13 +1545,25 @@ __global__ void k_lists_begin(unsigned long long *c, int force, unsigned few)
     }
 }
 
-// Whether the sums run over lists: the names hold the slots (uniform grid: 2^25 of them)
-// and the per-axis sweep, whose staging is its own, is off.
-bool lists_apply(const sph_ctx *ctx)
+// Whether the names hold the slots (uniform grid: 2^25 of them) and the per-axis sweep, whose
+// staging is its own, is off.
+bool lists_fit(const sph_ctx *ctx)
 {
-    if (ctx->lists.off || ctx->n <= 0) return false;
+    if (ctx->n <= 0) return false;
     if (ctx->adaptive) return true;
     return ctx->n <= ((int64_t)1 << kSlotBits) && !(ctx->p.flags & SPH_FLAG_AXIS_SWEEP);
+}
+
+// Whether the sums run over lists: as above, and there are arrays for them (ensure_lists).
+bool lists_apply(const sph_ctx *ctx)
+{
+    return lists_fit(ctx) && ctx->lists.pages && ctx->lists.cap >= ctx->cap;
+}
+
+// Pages a pool grows to: 512 names a particle on average, 2^32 in all.
+int64_t lists_most_pages(const sph_ctx *ctx)
+{
+    return std::min<int64_t>(16 * std::max<int64_t>(ctx->cap, 64), kMaxPages);
 }
 
 void free_lists(sph_ctx *ctx)
@@ -1567,14 +1579,31 @@ void free_lists(sph_ctx *ctx)
     P = ListPool();
 }
 
-// Arrays for the lists (never inside a capture): `pages` of them at least.  Where they would
-// take more than half of the device's free memory, which other allocations of the call may
-// need, the lists are switched off and the kernels of sph_pairs.cu run.
-int ensure_lists(sph_ctx *ctx, int64_t pages)
+// Arrays for the lists (never inside a capture): `pages` of them at least, five per particle to
+// start with, lists_most_pages at most.  Where they would take more than half of the memory
+// that is free once the present ones are given back, and which other allocations of the call
+// may need, they are not allocated: the pool at hand stays (false: it is smaller than asked
+// for), and a call that needs more than that, or has none, runs the kernels of sph_pairs.cu.
+bool ensure_lists(sph_ctx *ctx, int64_t pages)
 {
     ListPool &P = ctx->lists;
-    const int64_t cap = std::max<int64_t>(ctx->cap, 1);
-    pages = std::min<int64_t>(std::max<int64_t>(pages, 5 * cap + 1024), kMaxPages);
+    const int64_t cap = std::max<int64_t>(ctx->cap, 1), had = P.cap_pages;
+    pages = std::min(std::max<int64_t>(pages, 5 * cap + 1024), lists_most_pages(ctx));
+    const bool slots = P.cap < cap, more = had < pages;
+    if (!slots && !more) return true;
+    constexpr size_t kSlotBytes = 29, kPageBytes = 4 * (kPage + 1);
+    const size_t need = (slots ? kSlotBytes * (size_t)cap : 0) + (more ? kPageBytes * (size_t)pages : 0);
+    const size_t back = (slots ? kSlotBytes * (size_t)P.cap : 0) + (more ? kPageBytes * (size_t)had : 0);
+    size_t left = 0, total = 0;
+    if (cudaMemGetInfo(&left, &total) != cudaSuccess) {
+        cudaGetLastError();
+        left = 0;
+    }
+    if (ctx->limits.free_bytes >= 0) left = (size_t)ctx->limits.free_bytes;
+    if (need > (left + back) / 2) {
+        if (slots) free_lists(ctx);  // (of a smaller particle count)
+        return false;
+    }
     auto room = [&](auto **p, size_t bytes) {
         cudaFree(*p);
         *p = nullptr;
@@ -1582,28 +1611,23 @@ int ensure_lists(sph_ctx *ctx, int64_t pages)
         cudaGetLastError();  // (out of memory is not an error here)
         return false;
     };
+    auto pool = [&](int64_t n) {
+        P.cap_pages = n;
+        return room(&P.pages, sizeof(uint32_t) * kPage * (size_t)n) && room(&P.next, sizeof(int) * (size_t)n);
+    };
     bool ok = true;
-    if (P.cap < cap || P.cap_pages < pages) {
-        const size_t need = (P.cap < cap ? 29 * (size_t)cap : 0) +
-                            (P.cap_pages < pages ? 4 * (kPage + 1) * (size_t)pages : 0);
-        size_t left = 0, total = 0;
-        ok = cudaMemGetInfo(&left, &total) == cudaSuccess && need <= left / 2;
-    }
-    if (ok && P.cap < cap) {
+    if (slots) {
         ok = room(&P.head, sizeof(int) * cap) && room(&P.cnt, sizeof(int) * cap) &&
              room(&P.radius, sizeof(float) * cap) && room(&P.rows, 4 * sizeof(int) * cap) &&
              room(&P.mark, ((size_t)cap + 3) / 4 * 4);
         P.cap = cap;
     }
-    if (ok && P.cap_pages < pages) {
-        ok = room(&P.pages, sizeof(uint32_t) * kPage * (size_t)pages) && room(&P.next, sizeof(int) * (size_t)pages);
-        P.cap_pages = pages;
+    if (ok && more && !pool(pages)) {
+        ok = had > 0 && pool(had);  // (another process was quicker)
+        if (ok) return false;
     }
-    if (!ok) {
-        free_lists(ctx);
-        P.off = true;
-    }
-    return SPH_OK;
+    if (!ok) free_lists(ctx);
+    return ok;
 }
 
 static int list_grid(sph_ctx *ctx, int threads, int blocks_per_sm, int split = 1)

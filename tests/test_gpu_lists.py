@@ -8,7 +8,7 @@ import pytest
 
 from paper_1508_00115_gb300 import inputs
 
-from _gpu_util import check_density, check_force, force_pairs, oracle_state
+from _gpu_util import check_density, check_force, force_pairs, oracle_state, set_limit
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -164,3 +164,56 @@ def test_source_that_grows_past_a_capped_list_radius():
         kept += st["rebuilds"] == 0  # (a rebuild starts from the grown h)
         assert st["force_pairs"] == force_pairs(parts), k
     assert kept >= 3
+
+
+def _call(ctx, parts, factor):
+    """Build, density and force with every h scaled by factor; whether the sums ran over lists
+    (without them a pass evaluates a target once)."""
+    parts.t["h"] *= factor
+    ctx.build_cells(parts)
+    ctx.reset_stats()
+    ctx.density(parts)
+    st = ctx.stats()
+    ctx.force(parts)
+    return st["density_targets"] > parts.t["h"].numel() * st["density_passes"]
+
+
+def _check_call(ctx, parts):
+    g = parts.numpy()
+    g["perm"], g["ngb_hash"] = ctx.permutation(), ctx.ngb_hash()
+    s = oracle_state(g)
+    check_density(g, s)
+    check_force(g, s)
+
+
+@pytest.mark.parametrize("adaptive", [False, True])
+def test_pool_without_room_to_grow(adaptive):
+    """No device memory for a larger pool: the call that needs one runs without lists, and the
+    pool at hand serves those after it.  None for any pool: lists once there is."""
+    from paper_1508_00115_gb300 import binding
+    d = inputs.random_velocities(inputs.uniform(6000, seed=81), 0.3, 82)
+    flags = binding.SPH_FLAG_NGB_HASH | (binding.SPH_FLAG_ADAPTIVE if adaptive else 0)
+    ctx = binding.Context(6000, flags=flags)
+    parts = binding.Particles(d)
+    _call(ctx, parts, 1.0)
+    assert _call(ctx, parts, 0.98)
+    set_limit(ctx, 1, 0)
+    assert not _call(ctx, parts, 2.0)  # lists of 430 names: 14 pages, and the pool has 5 per particle
+    _check_call(ctx, parts)
+    assert _call(ctx, parts, 0.98)
+    _check_call(ctx, parts)
+    ctx = binding.Context(6000, flags=flags)
+    set_limit(ctx, 1, 0)
+    parts = binding.Particles(d)
+    _call(ctx, parts, 1.0)
+    assert not _call(ctx, parts, 0.98)
+    _check_call(ctx, parts)
+    ctx.steps(parts, 2, 1e-6)
+    set_limit(ctx, 1, -1)
+    _call(ctx, parts, 0.98)
+    assert _call(ctx, parts, 0.98)
+    ctx.steps(parts, 2, 1e-6)
+    ctx.build_cells(parts)
+    ctx.density(parts)
+    ctx.force(parts)
+    _check_call(ctx, parts)
