@@ -396,8 +396,8 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
         if (rc) return rc;
     }
     if (n > 0) {
-        if (lists_fit(ctx)) ensure_lists(ctx, 0);
-        int rc = density_begin(ctx, ctx->bin_mode);
+        const bool turn = lists_turn(ctx, 0);
+        int rc = density_begin(ctx, ctx->bin_mode, turn);
         if (rc) return rc;
         // passes without lists: every tile at first (and after a rebuild), then those with a
         // target left; individual time-steps: those with a target whose step ends
@@ -407,7 +407,8 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
         // names, walked by every Newton step: until a call has converged, passes without lists
         const bool settled = ctx->lists.settled || !ctx->adaptive;
         ctx->lists.settled = false;
-        bool use_lists = lists_apply(ctx) && settled;
+        bool use_lists = turn && settled;
+        bool fits = true;      // the lists fit the largest pool
         bool fresh = true;     // the next search is the first of the current cells
         bool again = false;    // ... of every target, at its present h
         bool some_done = false;  // a pass has run on the current cells
@@ -464,7 +465,7 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
                     const int64_t most = lists_most_pages(ctx), had = ctx->lists.cap_pages;
                     if ((ctx->h_counters[C_STALE] & 4ull) || had >= most ||
                         !ensure_lists(ctx, std::min(most, 2 * had))) {
-                        use_lists = false;
+                        use_lists = fits = false;
                     } else {
                         again = some_done;  // (those that are done keep a list for the force pass)
                         fresh = true;
@@ -508,10 +509,10 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
                 ctx->st.rebuilds++;
                 ++rebinned;
                 since = 0;
-                use_lists = lists_apply(ctx) && settled;
+                use_lists = turn && settled;
                 fresh = true;
                 again = some_done = partial = false;
-                rc = density_begin(ctx, ctx->bin_mode);  // slots were permuted
+                rc = density_begin(ctx, ctx->bin_mode, turn);  // slots were permuted
                 if (rc) return rc;
                 all_tiles = !ctx->bin_mode;
                 compact = ctx->bin_mode;
@@ -524,12 +525,13 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
         }
         rc = sync_h(ctx, parts);
         if (rc) return rc;
-        if (lists_apply(ctx)) {
+        ctx->lists.settled = unconv == 0;
+        if (turn && settled) lists_result(ctx, fits);
+        if (turn && lists_apply(ctx)) {
             // the force pass searches again where the lists at hand are not all there
             if (!use_lists || partial)
                 SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_STALE, 2, 1, ctx->stream));
             ctx->lists.ready = true;
-            ctx->lists.settled = unconv == 0;
             ctx->lists.stale = !use_lists || partial || (ctx->h_counters[C_STALE] & 3ull) != 0 || ctx->h_counters[C_GROWN] != 0;
         }
     }
@@ -867,7 +869,8 @@ static int do_step_bins(sph_ctx *ctx, sph_particles *parts, double dt_max, int l
 
 // flags of one step, ORed into C_GFLAGS: 1 = unconverged h, 2 = h beyond the cells,
 // 4 = h below what the uniform grid's FP32 frame resolves, 8 = a tensor-core wait of
-// the learned-h inference ran out
+// the learned-h inference ran out, 16 = the neighbour lists did not fit the pool (32: nor
+// would they a larger one)
 __global__ void k_step_flags(unsigned long long *c)
 {
     unsigned long long f = 0;
@@ -875,11 +878,12 @@ __global__ void k_step_flags(unsigned long long *c)
     if (c[C_HFLAG]) f |= 2ull;
     if (c[C_PREC]) f |= 4ull;
     if (c[C_TCERR]) f |= 8ull;
+    if (c[C_STALE] & 1ull) f |= c[C_STALE] & 4ull ? 48ull : 16ull;
     c[C_GFLAGS] |= f;
 }
 
 // One KDK step with no host synchronisation (the plan of the cell grids is fixed).
-static int graph_step(sph_ctx *ctx, sph_particles *parts, double dt, int passes)
+static int graph_step(sph_ctx *ctx, sph_particles *parts, double dt, int passes, bool lists)
 {
     int rc = dt > 0 ? set_dt(ctx, dt) : cfl_dt_device(ctx, parts);
     if (rc) return rc;
@@ -894,9 +898,8 @@ static int graph_step(sph_ctx *ctx, sph_particles *parts, double dt, int passes)
         rc = sync_h(ctx, parts);
         if (rc) return rc;
     }
-    rc = density_begin(ctx, false);
+    rc = density_begin(ctx, false, lists);
     if (rc) return rc;
-    const bool lists = lists_apply(ctx);
     ctx->lists.grow = kListGrow;
     if (lists) {
         rc = lists_begin(ctx, false);
@@ -998,14 +1001,13 @@ static int do_steps(sph_ctx *ctx, sph_particles *parts, int n_steps, double dt, 
         rc = tree_prepare_device(ctx, &tree_sig);
         if (rc) return rc;
     }
-    if (lists_fit(ctx)) {  // the pages the last searches took, and half as many again where there is room
-        rc = read_counters(ctx);
-        if (rc) return rc;
-        const int64_t used = (int64_t)ctx->h_counters[C_PAGES];
-        const bool more = used + used / 2 > ctx->lists.cap_pages;
-        if (more) ctx->lists.ready = false;
-        ensure_lists(ctx, more ? 2 * used : 0);
-    }
+    // the pages the last searches took, and half as many again where there is room
+    rc = read_counters(ctx);
+    if (rc) return rc;
+    const int64_t used = (int64_t)ctx->h_counters[C_PAGES];
+    const int64_t pages = std::max(used + used / 2 > ctx->lists.cap_pages ? 2 * used : 0, ctx->lists.want);
+    if (pages > ctx->lists.cap_pages) ctx->lists.ready = false;
+    const bool lists = lists_turn(ctx, pages);
     // capture one step on a private stream (the caller's may be the legacy default
     // stream, which cannot be captured); the graph is then launched on the caller's
     // stream.  The timing flag is suspended while capturing.  A graph captured for
@@ -1015,7 +1017,7 @@ static int do_steps(sph_ctx *ctx, sph_particles *parts, int n_steps, double dt, 
         if (rc) return rc;
     }
     sph_ctx::GraphKey key{*parts, dt > 0 ? dt : 0.0, ctx->n, ctx->grid.n_cells, ctx->grid.key_bits, passes, ctx->tile_w,
-                          tree_sig, ctx->sym_force, ctx->lists.pages, ctx->lists.cap_pages};
+                          tree_sig, ctx->sym_force, lists ? ctx->lists.pages : nullptr, lists ? ctx->lists.cap_pages : 0};
     if (!ctx->step_exec || !(key == ctx->graph_key)) {
         if (!ctx->cap_stream) SPH_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
         const uint32_t flags = ctx->p.flags;
@@ -1032,7 +1034,7 @@ static int do_steps(sph_ctx *ctx, sph_particles *parts, int n_steps, double dt, 
         const int64_t launches0 = ctx->st.kernel_launches;
         const int64_t passes0 = ctx->st.density_passes, fpasses0 = ctx->st.force_passes;
         ctx->tree.device_sized = ctx->adaptive;
-        rc = graph_step(ctx, parts, dt, passes);
+        rc = graph_step(ctx, parts, dt, passes, lists);
         ctx->tree.device_sized = false;
         ctx->graph_launches = ctx->st.kernel_launches - launches0;
         ctx->st.kernel_launches = launches0;  // capture launched nothing
@@ -1062,6 +1064,7 @@ static int do_steps(sph_ctx *ctx, sph_particles *parts, int n_steps, double dt, 
         ctx->g_keys64_alt = ctx->keys64_alt;
     }
     if (n_steps == 0) return SPH_OK;  // prepared: hydro, plan and graph are ready
+    ctx->lists.want = 0;
     const int64_t per_step = ctx->graph_launches;
     SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_FLOORS, 0, sizeof(unsigned long long), ctx->stream));
     SPH_CUDA(ctx, cudaMemsetAsync(ctx->counters + C_GFLAGS, 0, sizeof(unsigned long long), ctx->stream));
@@ -1098,6 +1101,14 @@ static int do_steps(sph_ctx *ctx, sph_particles *parts, int n_steps, double dt, 
         if (rc) return rc;
     }
     const unsigned long long gf = ctx->h_counters[C_GFLAGS];
+    if (lists) {
+        // a larger pool for the next call, or, where none is to be had, a step without lists
+        const int64_t had = ctx->lists.cap_pages;
+        const bool fitted = !(gf & 16ull);
+        const bool larger = !fitted && !(gf & 32ull) && had < lists_most_pages(ctx) && had >= pages;
+        if (larger) ctx->lists.want = 2 * had;
+        else lists_result(ctx, fitted);
+    }
     if (gf & 8ull) return fail(ctx, SPH_ERR_TIMEOUT, "predictor: a tensor-core wait ran out in a captured step");
     if (gf & 2ull) return fail(ctx, SPH_ERR_H_EXCEEDS_CELL, "some h grew beyond twice the planned cell side");
     if (gf & 1ull) return fail(ctx, SPH_ERR_NOT_CONVERGED, "smoothing lengths not converged in a captured step");
@@ -1519,11 +1530,12 @@ const char *sph_last_error(const sph_ctx *ctx)
 
 // For the tests, not declared in sph.h: let something of the context run out early, to reach
 // the calls' behaviour there.  which 0: the limiter's passes from now on; 1: the free device
-// memory (bytes) that the neighbour lists see.  value < 0: as it comes.
+// memory (bytes) that the neighbour lists see; 2: the pages of their largest pool.  value < 0: as
+// it comes.
 int sph_test_limit(sph_ctx *ctx, int32_t which, int64_t value)
 {
-    if (!ctx || which < 0 || which > 1) return SPH_ERR_INVALID_ARG;
-    (which == 0 ? ctx->limits.limiter_passes : ctx->limits.free_bytes) = value;
+    if (!ctx || which < 0 || which > 2) return SPH_ERR_INVALID_ARG;
+    (which == 0 ? ctx->limits.limiter_passes : which == 1 ? ctx->limits.free_bytes : ctx->limits.list_pages) = value;
     return SPH_OK;
 }
 

@@ -203,6 +203,11 @@ struct ListPool {
     int *rows = nullptr;        // 4 x cap: targets left by the last two passes, grown, dirty
     uint8_t *mark = nullptr;    // dirty targets of the present density call
     int64_t cap = 0, cap_pages = 0;
+    int64_t want = 0;           // pages that a captured step lacked
+    // calls in a row whose lists did not fit the largest pool, the calls still to go by without a
+    // search before one tries again, and the particle count of both
+    int misses = 0, skip = 0;
+    int64_t misses_n = 0;
     bool ready = false;         // lists of the current cells, from the last density call
     bool stale = false;         // ... that do not serve the force pass
     bool settled = false;       // the last density call converged
@@ -315,7 +320,7 @@ struct sph_ctx {
         int key_bits, passes, tile_w;
         uint64_t tree_sig;  // adaptive cells: arrays and capacities the captured build uses
         bool sym;           // symmetric force pass
-        const void *list_pages;  // neighbour-list pool
+        const void *list_pages;  // neighbour-list pool (null: a step without lists)
         int64_t list_cap;
         bool operator==(const GraphKey &o) const
         {
@@ -370,6 +375,7 @@ struct sph_ctx {
     struct {
         int64_t limiter_passes = -1;  // limiter passes left
         int64_t free_bytes = -1;      // device memory that is free for the lists
+        int64_t list_pages = -1;      // pages of the largest pool
     } limits;
 
     // statistics
@@ -450,7 +456,7 @@ int tree_read_device(sph_ctx *ctx);                             // sph_tree.cu (
 int tree_cell_keys_out(sph_ctx *ctx, int32_t *dev_keys);        // sph_tree.cu
 int tree_shrink_count(sph_ctx *ctx, sph_particles *parts);      // sph_tree.cu
 int tree_leaf_hcur(sph_ctx *ctx, sph_particles *parts);         // sph_tree.cu (before a force pass)
-int density_begin(sph_ctx *ctx, bool bins);                      // sph_pairs.cu
+int density_begin(sph_ctx *ctx, bool bins, bool lists);          // sph_pairs.cu
 // individual time-steps, sph_integrate.cu
 int bin_permute(sph_ctx *ctx, sph_particles *parts);  // after each permutation: bins, kept state, prediction
 int bin_active(sph_ctx *ctx, unsigned long long *n_active);  // active mask at ctx->bin_now (host read)
@@ -484,6 +490,8 @@ bool lists_fit(const sph_ctx *ctx);
 bool lists_apply(const sph_ctx *ctx);
 int64_t lists_most_pages(const sph_ctx *ctx);
 bool ensure_lists(sph_ctx *ctx, int64_t pages);  // (outside captures)
+bool lists_turn(sph_ctx *ctx, int64_t pages);    // (outside captures)
+void lists_result(sph_ctx *ctx, bool fitted);
 void free_lists(sph_ctx *ctx);
 int lists_begin(sph_ctx *ctx, bool force);
 unsigned list_few_rows(const sph_ctx *ctx);

@@ -1563,7 +1563,8 @@ bool lists_apply(const sph_ctx *ctx)
 // Pages a pool grows to: 512 names a particle on average, 2^32 in all.
 int64_t lists_most_pages(const sph_ctx *ctx)
 {
-    return std::min<int64_t>(16 * std::max<int64_t>(ctx->cap, 64), kMaxPages);
+    const int64_t most = std::min<int64_t>(16 * std::max<int64_t>(ctx->cap, 64), kMaxPages);
+    return ctx->limits.list_pages >= 0 ? std::min(most, ctx->limits.list_pages) : most;
 }
 
 void free_lists(sph_ctx *ctx)
@@ -1628,6 +1629,32 @@ bool ensure_lists(sph_ctx *ctx, int64_t pages)
     }
     if (!ok) free_lists(ctx);
     return ok;
+}
+
+// Whether a density call (or a captured step) searches into lists; `pages` as in ensure_lists.
+// Lists that do not fit the largest pool cost a search of no use in every call (adaptive sets of
+// more than 40 M particles, whose names would take more than 2^32, and lists beyond 512 names a
+// particle): after two such calls in a row the next goes by without, after three the next two,
+// then 4, 8, ... up to 64 before one tries again.
+bool lists_turn(sph_ctx *ctx, int64_t pages)
+{
+    ListPool &P = ctx->lists;
+    if (!lists_fit(ctx)) return false;
+    if (P.misses_n != ctx->n) P.misses = P.skip = 0;
+    if (P.skip > 0) {
+        --P.skip;
+        return false;
+    }
+    ensure_lists(ctx, pages);
+    return lists_apply(ctx);
+}
+
+void lists_result(sph_ctx *ctx, bool fitted)
+{
+    ListPool &P = ctx->lists;
+    P.misses = fitted ? 0 : std::min(P.misses + 1, 8);
+    P.skip = P.misses < 2 ? 0 : 1 << (P.misses - 2);
+    P.misses_n = ctx->n;
 }
 
 static int list_grid(sph_ctx *ctx, int threads, int blocks_per_sm, int split = 1)

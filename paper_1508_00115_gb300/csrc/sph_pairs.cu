@@ -1983,11 +1983,11 @@ __global__ void k_density_begin(uint8_t *__restrict__ active, const uint8_t *__r
     if (mark) mark[i] = 0;
 }
 
-// bins: the particles whose step ends now (individual time-steps)
-int density_begin(sph_ctx *ctx, bool bins)
+// bins: the particles whose step ends now (individual time-steps); lists: the call has lists
+int density_begin(sph_ctx *ctx, bool bins, bool lists)
 {
     const int n = (int)ctx->n;
-    uint8_t *mark = lists_apply(ctx) ? ctx->lists.mark : nullptr;
+    uint8_t *mark = lists ? ctx->lists.mark : nullptr;
     k_density_begin<<<(unsigned)std::max(1, (n + 255) / 256), 256, 0, ctx->stream>>>(
         ctx->active, bins ? ctx->bin_active : nullptr, ctx->h_lo, ctx->h_hi, mark, n, ctx->counters);
     SPH_LAUNCH(ctx, "density begin");

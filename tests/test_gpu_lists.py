@@ -217,3 +217,59 @@ def test_pool_without_room_to_grow(adaptive):
     ctx.density(parts)
     ctx.force(parts)
     _check_call(ctx, parts)
+
+
+@pytest.mark.parametrize("adaptive", [False, True])
+@pytest.mark.parametrize("pages", [1.0, 2.0, 2.5, 3.0, 3.5, 4.0, 5.0])
+def test_pool_that_runs_out(adaptive, pages):
+    """Pools of too few pages per particle: they run out in the first search, in that of the
+    targets whose h left its list, in that of a grown neighbour's, or not, outside captures and
+    inside them; the sums are the same."""
+    from paper_1508_00115_gb300 import binding
+    n = 3000
+    d = inputs.random_velocities(inputs.uniform(n, seed=91), 0.3, 92)
+    flags = binding.SPH_FLAG_NGB_HASH | (binding.SPH_FLAG_ADAPTIVE if adaptive else 0)
+    ctx = binding.Context(n, flags=flags, cell_factor=1.25)
+    set_limit(ctx, 2, int(pages * n))
+    parts = binding.Particles(d)
+    for k, share in enumerate((0.0, 1.0, 0.03, 0.3, 0.03)):
+        _lowered(parts, share, 0.9, 93 + k)
+        ctx.build_cells(parts)
+        ctx.density(parts)
+        ctx.force(parts)
+        _check_call(ctx, parts)
+    for k in range(3):
+        ctx.steps(parts, 2, 1e-4)
+        ctx.build_cells(parts)
+        ctx.density(parts)
+        ctx.force(parts)
+        _check_call(ctx, parts)
+
+
+def test_lists_that_never_fit():
+    """Lists that do not fit the largest pool: the search that shows it runs in ever fewer of
+    the calls, and captured steps are captured again without it."""
+    from paper_1508_00115_gb300 import binding
+    n = 3000
+    d = inputs.random_velocities(inputs.uniform(n, seed=95), 0.3, 96)
+    ctx = binding.Context(n)
+    set_limit(ctx, 2, n)
+    parts = binding.Particles(d)
+    launches = []
+    for _ in range(17):
+        parts.t["h"] *= 0.98
+        ctx.build_cells(parts)
+        ctx.reset_stats()
+        ctx.density(parts)
+        launches.append(ctx.stats()["kernel_launches"])
+    tried = [v > min(launches) for v in launches]
+    assert [k for k, t in enumerate(tried) if t] == [0, 1, 3, 6, 11], launches
+    ctx = binding.Context(n)
+    set_limit(ctx, 2, n)
+    parts = binding.Particles(d)
+    steps = []
+    for _ in range(4):
+        ctx.reset_stats()
+        ctx.steps(parts, 3, 1e-6)
+        steps.append(ctx.stats()["kernel_launches"])
+    assert steps[1] == steps[3] < steps[2], steps  # (the first call's hydro pass has missed once)
