@@ -82,6 +82,8 @@ static void free_particles(sph_ctx *c)
 static int alloc_particles(sph_ctx *c, int64_t cap)
 {
     free_particles(c);
+    if (c->step_exec) cudaGraphExecDestroy(c->step_exec);  // (it holds the arrays that were freed)
+    c->step_exec = nullptr;
     cap = std::max<int64_t>(cap, 1);
     const int64_t sort_tiles = std::max<int64_t>((cap + 4095) / 4096, 128);  // (kRsRowTiles short tiles)
     c->tile_cap = cap + cap / kMinTile + 64;

@@ -1,5 +1,7 @@
 """The cell build's sort and prefix sums at the edges of their tiles: permutation and keys
 equal a stable argsort of the keys of the input order, exactly."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -62,3 +64,26 @@ def test_device_sized_trees_step_like_host_built_ones(n, leaf):
         out.append((parts.numpy(), ctx.permutation()))
         ctx.close()
     _same_state(out[0][0], out[1][0], out[0][1], out[1][1], _RT_STEPS, _RT_RHO)
+
+
+@pytest.mark.parametrize("adaptive", [False, True])
+def test_captured_steps_after_the_scratch_was_replaced(adaptive):
+    """A context that grows to more particles and comes back replays nothing that it captured with
+    the arrays it had before."""
+    n = 1500
+    d = inputs.random_velocities(inputs.uniform(n, seed=7), 0.2, 8)
+    out = []
+    for grow in (False, True):
+        ctx = binding.Context(n, flags=binding.SPH_FLAG_ADAPTIVE if adaptive else 0)
+        parts = binding.Particles(d)
+        ctx.steps(parts, 2, 1e-5)
+        if grow:
+            for m in (4 * n, n):
+                assert binding.lib().sph_set_n(ctx.h, ctypes.c_int64(m)) == binding.SPH_OK
+        else:
+            ctx.build_cells(parts)  # (as a new particle count does, the next call starts with a hydro pass)
+        ctx.steps(parts, 2, 1e-5)
+        out.append(parts.numpy())
+        ctx.close()
+    for k in ("x", "vx", "u", "h", "rho", "ax"):
+        assert np.array_equal(np.sort(out[0][k]), np.sort(out[1][k])), k
