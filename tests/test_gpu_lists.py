@@ -273,3 +273,17 @@ def test_lists_that_never_fit():
         ctx.steps(parts, 3, 1e-6)
         steps.append(ctx.stats()["kernel_launches"])
     assert steps[1] == steps[3] < steps[2], steps  # (the first call's hydro pass has missed once)
+
+
+@pytest.mark.parametrize("n,factor", [(1200, 1.3), (4000, 1.35), (4000, 1.5), (4000, 2.0), (6000, 2.4)])
+def test_guesses_above_the_root(n, factor):
+    """First calls whose guess asks for more names than the pool holds: passes without lists
+    until the lists will be short, then one search for all."""
+    from paper_1508_00115_gb300 import binding
+    d = inputs.random_velocities(inputs.uniform(n, seed=101), 0.3, 102)
+    ctx = binding.Context(n, flags=binding.SPH_FLAG_NGB_HASH)
+    parts = binding.Particles(d)
+    _call(ctx, parts, factor)
+    _check_call(ctx, parts)
+    assert _call(ctx, parts, 0.97)
+    _check_call(ctx, parts)
