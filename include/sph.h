@@ -279,11 +279,14 @@ int sph_build_cells(sph_ctx *ctx, sph_particles *parts);
  * |N_w/N_ngb - 1| <= h_tol -- or their bracket is narrower than 2^-21 h, the
  * resolution of the FP32 sums -- or max_h_iter evaluations ran since the last
  * re-binning.  A pass searches each target's neighbours once, a little beyond h, into a
- * list and iterates on it; only targets whose h leaves that radius need another pass.  Rebuilds the cells (permuting the arrays again, restarting the
- * iteration) if some h outgrows its cell, at most 8 times per call
- * (SPH_ERR_NOT_CONVERGED beyond that).
- * Writes h, rho, P, c, f, divv, curl, n_ngb.  *iters_out (may be NULL) = passes
- * run.  Requires sph_build_cells on the current positions.  Host read: the
+ * list and iterates on it; only targets whose h leaves that radius need another pass.
+ * (Without lists -- the axis sweep, uniform grids of more than 2^25 particles, adaptive
+ * contexts until a call has converged, no room -- a pass is one evaluation.)  Rebuilds
+ * the cells (permuting the arrays again, restarting the iteration) if some h outgrows
+ * its cell, at most 32 times per call (SPH_ERR_NOT_CONVERGED beyond that).
+ * Writes h, rho, P, c, f, divv, curl, n_ngb.  *iters_out (may be NULL) = evaluations
+ * of the target that took most (where targets were searched for again, at most that
+ * many).  Requires sph_build_cells on the current positions.  Host read: the
  * count of targets left after each pass.  On the uniform grid, SPH_ERR_PRECISION if a
  * converged h is below cell side / SPH_FRAME_RATIO (results are written, and the
  * state counts as having densities, so that sph_force may follow). */

@@ -385,8 +385,9 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
 {
     if (!ctx->built) return fail(ctx, SPH_ERR_STATE, "sph_density needs sph_build_cells on the current positions");
     int n = (int)ctx->n;
-    int iters = 0;     // passes
-    int since = 0;     // evaluations since the last re-binning (each restarts the iteration)
+    int iters = 0;     // evaluations of the target that took most
+    int since = 0;     // ... since the last re-binning (each restarts the iteration), of those left
+    int before = 0;    // ... before it
     int rebinned = 0;  // re-binnings in this call
     unsigned long long unconv = 0;
     if (n > 0 && (ctx->p.flags & SPH_FLAG_AUTOTUNE) && !ctx->tuned) {
@@ -492,13 +493,15 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
                 }
                 some_done = true;
                 lost = lost0 + ctx->h_counters[C_LOST];
-                since += (int)ctx->h_counters[C_PASS + 4 * (pass - 1) + 3];
+                const unsigned long long evals = ctx->h_counters[C_PASS + 4 * (pass - 1) + 3];
+                iters = std::max(iters, before + since + (int)(evals >> 32));
+                since += (int)(unsigned)evals;
                 unconv = ctx->h_counters[C_PASS + 4 * (pass - 1)];
             } else {
                 ++since;
+                iters = std::max(iters, before + since);
                 unconv = ctx->h_counters[C_UNCONV];
             }
-            ++iters;
             if (unconv == 0 || last) break;
             // adaptive: lists much longer than the current h need (1 leaf in 16); the sums over
             // neighbour lists iterate to the end, so that few are left to gain from new cells
@@ -526,6 +529,7 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
                 if (rc) return rc;
                 ctx->st.rebuilds++;
                 ++rebinned;
+                before = iters;
                 since = 0;
                 use_lists = turn && settled;
                 fresh = true;
@@ -570,7 +574,7 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
     ctx->hydro_valid = false;
     if (unconv) {
         char buf[160];
-        snprintf(buf, sizeof buf, "%llu smoothing lengths not converged after %d passes", unconv, iters);
+        snprintf(buf, sizeof buf, "%llu smoothing lengths not converged after %d evaluations", unconv, iters);
         return fail(ctx, SPH_ERR_NOT_CONVERGED, buf);
     }
     if (n > 0 && ctx->h_counters[C_PREC]) {

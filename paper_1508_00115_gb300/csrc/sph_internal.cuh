@@ -76,7 +76,8 @@ enum Counter {
     C_LOST = 32,      // targets that used up their evaluations without converging
     C_FTICKET = 33,   // list sums of the force pass: tickets of the search and of the sums
     C_PASS = 35,      // list sums, four per density pass: targets that need another pass, tickets
-                      // of the search and of the sums, most evaluations of a target left
+                      // of the search and of the sums, most evaluations of a target (in the low
+                      // half of those left, in the high half of all)
     C_GROWN = C_PASS + 4 * 8,  // neighbour lists: targets whose h outgrew the radius their
                                // neighbours searched with
     C_DIRTY,                   // ... and the targets among those neighbours that miss them

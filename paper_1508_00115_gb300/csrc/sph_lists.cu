@@ -833,7 +833,8 @@ struct DensityListArgs {
     const unsigned long long *__restrict__ n_rows;
     const int *__restrict__ leaf_of;
     int nb;
-    unsigned long long *left;  // targets that need another pass ([3]: most evaluations of one of them)
+    // targets that need another pass ([3], in two halves: most evaluations of one of them, of any)
+    unsigned long long *left;
     int *left_rows;            // ... and which
     int *grown_rows;           // targets whose h outgrew the radius their neighbours searched with
     int budget;      // evaluations of a target in this pass
@@ -1078,7 +1079,7 @@ __global__ void __launch_bounds__(kSumThreads, kSumBlocks) k_density_l(DensityLi
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     const int ntiles = *a.s.n_tiles;
     unsigned long long acc_pairs = 0ull;
-    unsigned acc_targets = 0u, acc_lost = 0u, acc_flag = 0u, left_ev = 0u;
+    unsigned acc_targets = 0u, acc_lost = 0u, acc_flag = 0u, left_ev = 0u, most_ev = 0u;
     unsigned *ticket = reinterpret_cast<unsigned *>(a.s.ticket);
     unsigned tk = 0u;
     if (lane == 0) tk = atomicAdd(ticket, 1u);
@@ -1269,18 +1270,21 @@ __global__ void __launch_bounds__(kSumThreads, kSumBlocks) k_density_l(DensityLi
             }
             todo = __ballot_sync(kFull, run);
         }
+        most_ev = max(most_ev, (unsigned)ev);
     }
     const unsigned long long tp = warp_sum_ull(acc_pairs);
     const unsigned tt = __reduce_add_sync(kFull, acc_targets);
     const unsigned tf = __reduce_or_sync(kFull, acc_flag);
     const unsigned tl = __reduce_max_sync(kFull, left_ev), tx = __reduce_add_sync(kFull, acc_lost);
+    const unsigned tm = __reduce_max_sync(kFull, most_ev);
     if (lane == 0) {
         unsigned long long *c = a.s.counters;
         if (tp) atomicAdd(c + C_DPAIRS, tp);
         if (tt) atomicAdd(c + C_DTARGETS, (unsigned long long)tt);
         if (tf & 2u) atomicOr(c + C_HFLAG, 1ull);
         if (tf & 4u) atomicOr(c + C_PREC, 1ull);
-        if (tl) atomicMax(a.left + 3, (unsigned long long)tl);
+        if (tl) atomicMax(reinterpret_cast<unsigned *>(a.left + 3), tl);
+        if (tm) atomicMax(reinterpret_cast<unsigned *>(a.left + 3) + 1, tm);
         if (tx) atomicAdd(c + C_LOST, (unsigned long long)tx);
     }
 }

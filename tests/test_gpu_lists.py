@@ -287,3 +287,22 @@ def test_guesses_above_the_root(n, factor):
     _check_call(ctx, parts)
     assert _call(ctx, parts, 0.97)
     _check_call(ctx, parts)
+
+
+@pytest.mark.parametrize("factor", [0.7, 0.9, 0.99, 1.1])
+def test_iterations_are_evaluations(factor):
+    """sph_density reports the evaluations of the h iteration, as many with lists, which iterate
+    within a pass, as without (no room for them): one may differ where a target ends at h_tol."""
+    from paper_1508_00115_gb300 import binding
+    d = inputs.uniform(6000, seed=111)
+    its = []
+    for free in (-1, 0):
+        ctx = binding.Context(6000, cell_factor=1.5)
+        set_limit(ctx, 1, free)
+        parts = binding.Particles(d)
+        ctx.build_cells(parts)
+        ctx.density(parts)
+        parts.t["h"] *= factor
+        ctx.build_cells(parts)
+        its.append(ctx.density(parts))
+    assert its[1] >= 2 and abs(its[0] - its[1]) <= 1, its
