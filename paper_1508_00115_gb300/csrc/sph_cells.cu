@@ -995,7 +995,7 @@ constexpr int kAxisWarps = 4;
 
 // one warp per cell: projections (cell-relative FP32 positions, unit directions) and
 // their ranks (ties by slot); a cell too large for the shared buffer is written in
-// slot order with projections -inf, so that no sweep stops inside it
+// slot order with projections NaN, which no sweep in either direction drops
 __global__ void __launch_bounds__(32 * kAxisWarps) k_axis_sort(const int *__restrict__ cs, int64_t ncells,
                                                                 const float4 *__restrict__ pos4, int64_t cap,
                                                                 float2 *__restrict__ axis)
@@ -1010,7 +1010,7 @@ __global__ void __launch_bounds__(32 * kAxisWarps) k_axis_sort(const int *__rest
         const float inv = rsqrtf(dx * dx + dy * dy + dz * dz);
         float2 *out = axis + (size_t)d * cap + b;
         if (cnt > kAxisMax) {
-            for (int k = lane; k < cnt; k += 32) out[k] = make_float2(-INFINITY, __int_as_float(b + k));
+            for (int k = lane; k < cnt; k += 32) out[k] = make_float2(__int_as_float(0x7fffffff), __int_as_float(b + k));
             continue;
         }
         for (int k = lane; k < cnt; k += 32) {

@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(kPairThreads, kDensityBlocks) k_density(Densit
             if (SWEEP && sw_d >= 0 && v) {
                 const float2 e = a.axis[(size_t)sw_d * a.axis_stride + bs + (sw_sg > 0.f ? q : be - bs - 1 - q)];
                 j = __float_as_int(e.y);
-                v = sw_sg * e.x < sw_lim;
+                v = !(sw_sg * e.x >= sw_lim);  // (NaN: a cell without an order)
             }
         };
         // software pipeline: the positions of the next chunk are loaded before the
@@ -1211,7 +1211,7 @@ __global__ void __launch_bounds__(kPairThreads, MODE == 1 ? kForceBlocks : kForc
                 if (SWEEP && sw_d >= 0 && vq) {  // the cell's order along the axis, up to the sweep bound
                     const float2 e = a.axis[(size_t)sw_d * a.axis_stride + bs + (sw_sg > 0.f ? q : be - bs - 1 - q)];
                     j = __float_as_int(e.y);
-                    vq = sw_sg * e.x < sw_lim;
+                    vq = !(sw_sg * e.x >= sw_lim);  // (NaN: a cell without an order)
                 }
                 // (no branch: a lane past the chunk's end reads slot 0 and keeps nothing)
                 const int jj = vq ? j : 0;

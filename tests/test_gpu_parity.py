@@ -367,6 +367,18 @@ def test_axis_sweep_parity(tw):
         ctx.step(parts, 2e-4)
 
 
+def test_axis_sweep_of_cells_without_an_order():
+    """Cells of more than 256 particles are not sorted along the axes: every source of theirs is
+    tested, whichever side of the target's cell they lie on."""
+    from paper_1508_00115_gb300 import binding
+    d = _uniform_moving(7000, 34)
+    ctx, parts, g = gpu_hydro(d, flags=binding.SPH_FLAG_NGB_HASH | binding.SPH_FLAG_AXIS_SWEEP, cell_factor=2.5)
+    assert np.bincount(ctx.cell_keys()).max() > 256 > np.bincount(ctx.cell_keys()).min()
+    s = oracle_state(g)
+    check_density(g, s)
+    check_force(g, s)
+
+
 @pytest.mark.parametrize("pin,adaptive", [(True, False), (False, False), (True, True)])
 def test_step_host_matches_device_step(pin, adaptive):
     """sph_step_host (host arrays, copies inside the call -- the results go back on a
