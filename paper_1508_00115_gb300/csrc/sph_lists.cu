@@ -40,6 +40,7 @@ constexpr int kSumThreads = 128;
 constexpr int kSumBlocks = 5;
 constexpr int kSearchF4 = 352 + 2 * kCodes / 16;  // float4 of shared memory per searching warp
 constexpr int kPage = 32;         // names per page
+static_assert(kMaxPages * kPage <= (int64_t)1 << 32, "positions in the pool are 32 bits");
 constexpr int kSlotBits = 25;     // uniform grid: bits of a name that hold the slot
 
 // ------------------------------------------- candidate search on the tensor cores
@@ -323,8 +324,9 @@ __device__ __forceinline__ void emit_batch(const SearchArgs &a, const unsigned (
         }
         if (R.dead) return;  // warp-uniform
         const int fresh = (int)base + incl - np;
-        dst[lane] = make_uint4((unsigned)(R.chunk * kPage + R.fill - R.start - off[lane]),
-                               (unsigned)(fresh * kPage - room - off[lane]), (unsigned)(off[lane] + room), 0u);
+        // (positions are 32 bits without a sign: modulo 2^32, as the pool has 2^32 names at most)
+        dst[lane] = make_uint4((unsigned)R.chunk * kPage + (unsigned)(R.fill - R.start - off[lane]),
+                               (unsigned)fresh * kPage - (unsigned)(room + off[lane]), (unsigned)(off[lane] + room), 0u);
         if (np > 0) {
             if (R.fill == 0) R.first = fresh;
             else a.next[R.chunk + 1] = fresh;
