@@ -362,11 +362,11 @@ static int radix_pass(sph_ctx *ctx, const K *kin, const uint32_t *vin, K *kout, 
 {
     constexpr int kTile = kRsThreads * ITEMS;
     constexpr size_t smem = (size_t)kTile * (sizeof(K) + sizeof(uint32_t));
-    static bool optin = false;  // (per function, once per process)
-    if (!optin) {
+    constexpr int kInstance = (sizeof(K) == 8 ? 4 : 0) + (!ROWS ? 3 : ITEMS == 4 ? 0 : ITEMS == 8 ? 1 : 2);
+    if (!(ctx->optin & kOptSort << kInstance)) {
         SPH_CUDA(ctx, cudaFuncSetAttribute(k_radix_scatter_c<K, ITEMS, ROWS>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        optin = true;
+        ctx->optin |= kOptSort << kInstance;
     }
     const int ntiles = (n + kTile - 1) / kTile;
     k_radix_hist<K, ITEMS, ROWS><<<ntiles, kRsThreads, 0, ctx->stream>>>(kin, n, shift, ctx->hist, ntiles);

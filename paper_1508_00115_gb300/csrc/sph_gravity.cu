@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kGravThreads, kGravBlocks) k_gravity(GravArgs 
 template <bool SOFT>
 static int launch_gravity(sph_ctx *ctx, const GravArgs &a)
 {
-    static int blocks_per_sm = 0;  // occupancy of this instantiation (per process)
+    int &blocks_per_sm = ctx->grav_blocks[SOFT];  // occupancy of this instantiation
     if (blocks_per_sm == 0) {
         SPH_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_gravity<SOFT>, kGravThreads,
                                                                     0));

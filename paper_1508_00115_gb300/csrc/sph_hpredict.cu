@@ -997,10 +997,9 @@ int hp_collect(sph_ctx *ctx, sph_particles *parts)
 
 static int hp_smem_optin(sph_ctx *ctx, size_t bytes)
 {
-    static bool done = false;
-    if (done) return SPH_OK;
+    if (ctx->optin & kOptTrain) return SPH_OK;
     SPH_CUDA(ctx, cudaFuncSetAttribute(k_hp_train_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    done = true;
+    ctx->optin |= kOptTrain;
     return SPH_OK;
 }
 

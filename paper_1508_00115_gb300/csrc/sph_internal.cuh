@@ -372,6 +372,11 @@ struct sph_ctx {
 
     sph::ListPool lists;  // neighbour lists
 
+    // kernels that this context has opted into more than 48 KB of shared memory (an attribute of
+    // the function on the context's device), and gravity blocks per SM, unsoftened and softened
+    unsigned optin = 0;
+    int grav_blocks[2] = {0, 0};
+
     // what runs out where the tests want it to (sph_test_limit); below 0: no limit
     struct {
         int64_t limiter_passes = -1;  // limiter passes left
@@ -403,6 +408,9 @@ int cuda_fail(sph_ctx *ctx, cudaError_t e, const char *what);
         cudaError_t e_ = cudaGetLastError();                          \
         if (e_ != cudaSuccess) return sph::cuda_fail(ctx, e_, what);  \
     } while (0)
+
+// bits of sph_ctx::optin; the cell sort's instances from kOptSort on
+constexpr unsigned kOptPairs = 1u, kOptTrain = 2u, kOptSort = 4u;
 
 // prefix sums over a warp and a block
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v)

@@ -1733,21 +1733,7 @@ static SumArgs sum_args(sph_ctx *ctx, sph_particles *parts)
 }
 
 constexpr size_t kSearchSmem = (kListThreads / 32) * (16 * (size_t)kSearchF4 + 4 * 33);
-
-// Opt the searches into more than 48 KB of dynamic shared memory (once per process; the
-// attribute is per function, not per device).
-static int search_optin(sph_ctx *ctx)
-{
-    static bool done = false;
-    if (done) return SPH_OK;
-    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    SPH_CUDA(ctx, cudaFuncSetAttribute(k_search<0, kSearchFew>, at, (int)kSearchSmem));
-    SPH_CUDA(ctx, cudaFuncSetAttribute(k_search<0, kSearchMany>, at, (int)kSearchSmem));
-    SPH_CUDA(ctx, cudaFuncSetAttribute(k_search<1, kSearchFew>, at, (int)kSearchSmem));
-    SPH_CUDA(ctx, cudaFuncSetAttribute(k_search<1, kSearchMany>, at, (int)kSearchSmem));
-    done = true;
-    return SPH_OK;
-}
+static_assert(kSearchSmem <= 48 * 1024, "no opt-in needed");
 
 // Pass `pass` (below kListPasses) of a density call: lists for the active targets; a pass
 // after the first runs only if the one before left targets.  pass < 0: the force pass's own
@@ -1756,8 +1742,6 @@ int run_search(sph_ctx *ctx, sph_particles *parts, int pass, bool all)
 {
     const ListPool &P = ctx->lists;
     const bool force = pass < 0;
-    const int rc = search_optin(ctx);
-    if (rc) return rc;
     SearchArgs a{};
     a.pos4 = ctx->pos4;
     a.h = parts->h;

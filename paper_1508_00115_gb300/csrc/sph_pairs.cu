@@ -1674,12 +1674,10 @@ static size_t force_sym_smem()
     return slots * (4 * sizeof(float4) + sizeof(int) + sizeof(float));
 }
 
-// Opt the pair kernels into more than 48 KB of dynamic shared memory (once per process;
-// the attribute is per function, not per device).
+// Opt the pair kernels into more than 48 KB of dynamic shared memory.
 static int smem_optin(sph_ctx *ctx)
 {
-    static bool done = false;
-    if (done) return SPH_OK;
+    if (ctx->optin & kOptPairs) return SPH_OK;
     const int d16 = (int)density_smem<16>(true), d32 = (int)density_smem<32>(true);
     const int f16 = (int)force_smem<16>(true), f32 = (int)force_smem<32>(true);
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
@@ -1695,7 +1693,7 @@ static int smem_optin(sph_ctx *ctx)
     SPH_OPT_D(2)
 #undef SPH_OPT_D
     SPH_CUDA(ctx, cudaFuncSetAttribute(k_force_sym, at, (int)force_sym_smem()));
-    done = true;
+    ctx->optin |= kOptPairs;
     return SPH_OK;
 }
 

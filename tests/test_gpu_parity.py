@@ -405,3 +405,36 @@ def test_step_host_matches_device_step(pin, adaptive):
     for key in gd:
         assert np.array_equal(gd[key], gh[key]), key
     assert np.array_equal(ctx_d.permutation(), ctx_h.permutation())
+
+
+def test_contexts_of_several_threads():
+    """A context per thread, each on its own stream and from its own sizes, all at once: bit for
+    bit what each gives alone (nothing is set up once for the process)."""
+    import threading
+    from paper_1508_00115_gb300 import binding
+    sizes = (700, 5000, 140000, 20000)
+
+    def run(n, out, k):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            flags = binding.SPH_FLAG_ADAPTIVE if k % 2 else 0
+            ctx = binding.Context(n, stream=stream.cuda_stream, flags=flags)
+            parts = binding.Particles(_uniform_moving(n, 50 + k))
+            ctx.step(parts, 1e-4)
+            ctx.steps(parts, 2, 1e-4)
+            if not flags:
+                ctx.gravity(1.0, 0.01)
+            out[k] = parts.numpy()
+            ctx.close()
+
+    alone, together = {}, {}
+    for k, n in enumerate(sizes):
+        run(n, alone, k)
+    threads = [threading.Thread(target=run, args=(n, together, k)) for k, n in enumerate(sizes)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for k in range(len(sizes)):
+        for key in alone[k]:
+            assert np.array_equal(alone[k][key], together[k][key]), (k, key)
