@@ -897,13 +897,13 @@ __device__ __forceinline__ unsigned sort_rows(unsigned key)
     return key;
 }
 
-// 1/sqrt(x) and 1/x as one MUFU instruction each; a separation of zero (or whose square is
-// denormal) gives 0
+// 1/sqrt(x), 0 for a separation of zero (a denormal square is one of pairs that are separated:
+// three more instructions for its scaling); 1/x as one MUFU instruction
 __device__ __forceinline__ float inv_sqrt(float x)
 {
     float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return x > 1.2e-38f ? y : 0.f;
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return x > 0.f ? y : 0.f;
 }
 __device__ __forceinline__ float inv(float x)
 {

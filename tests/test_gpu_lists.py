@@ -306,3 +306,33 @@ def test_iterations_are_evaluations(factor):
         ctx.build_cells(parts)
         its.append(ctx.density(parts))
     assert its[1] >= 2 and abs(its[0] - its[1]) <= 1, its
+
+
+def test_pairs_closer_than_normal_squares():
+    """Two particles 3e-20 apart (at a cell centre of a box of side 1e-3), whose squared distance
+    is a denormal FP32 number, approach each other: the pair has its direction, and its signal
+    velocity counts."""
+    from paper_1508_00115_gb300 import binding
+    n, box = 4000, 1e-3
+    d = inputs.random_velocities(inputs.uniform(n, seed=121, box=box), 0.1, 122)
+    nc = None
+    for _ in range(2):
+        ctx = binding.Context(n, box_size=box, flags=binding.SPH_FLAG_NGB_HASH)
+        parts = binding.Particles(d)
+        ctx.build_cells(parts)
+        ctx.density(parts)
+        ctx.force(parts)
+        st, g = ctx.stats(), parts.numpy()
+        g["perm"], g["ngb_hash"] = ctx.permutation(), ctx.ngb_hash()
+        if nc is None:
+            nc = st["nc"]
+            c = 0.5 * (box / nc)
+            for k in "xyz":
+                d[k][:2] = c
+            d["x"][1] = c + 2 * np.spacing(c)
+            d["vx"][:2] = (5.0, -5.0)
+    assert st["nc"] == nc and 0 < (d["x"][1] - d["x"][0]) ** 2 < 1.1e-38
+    s = oracle_state(g, box)
+    check_density(g, s)
+    check_force(g, s)
+    assert (g["vsig"][g["perm"] < 2] > 30).all()
