@@ -509,11 +509,13 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
             const bool shrunk = ctx->adaptive && !few_left && ctx->h_counters[C_SHRINK] * 16 > (unsigned long long)ctx->tree.n_leaves;
             const bool outgrown = ctx->h_counters[C_HFLAG] != 0;
             // where many h grew, the lists of their neighbours miss them, and the force pass would
-            // search for everything once more: do that now (from a guessed h, an eighth left after
-            // the first pass: 2 M clustered 19.1 -> 17.6 ms, 200,000 uniform 1.25 -> 1.16 ms,
-            // 20,000 clustered 1.57 -> 1.52 ms; 32,768 uniform 0.50 -> 0.52 ms, where a search of
-            // the eighth is quick and the force pass's own, at h itself, gives it shorter lists)
-            const unsigned long long many = ctx->adaptive || n >= 100000 ? list_few_rows(ctx) : (unsigned long long)n / 3;
+            // search for everything once more: do that now.  On small uniform sets a search of an
+            // eighth is quick, and the force pass's own, at h itself, gives it shorter lists.  (A
+            // density and a force pass from a guessed h that leaves an eighth after the first pass,
+            // us, again from n / 24 left on and from n / 3 on: uniform 20,000 496, 491; 32,768 510,
+            // 495; 50,000 574, 565; 80,000 723, 747; 200,000 1,152, 1,225; 2 M 7,675, 7,986; clustered
+            // 5,000 1,156, 1,164; 20,000 1,487, 1,564; 80,000 3,726, 3,676; 2 M 15,032, 18,159)
+            const unsigned long long many = ctx->adaptive || n >= 65536 ? list_few_rows(ctx) : (unsigned long long)n / 3;
             again = use_lists && !partial && !ctx->sym_force && unconv > many;
             if (outgrown && rebinned >= kMaxRebins) {
                 char buf[160];

@@ -27,10 +27,9 @@ namespace sph {
 
 constexpr int kCodes = 1024;      // hits of a batch written out at once
 constexpr int kListThreads = 128;
-// resident blocks per SM the search is compiled for: more warps where there are tiles for all of
-// them many times over, else more registers for each (ms per call with 5 and with 7: 512 boxes
-// of 37 k 154.3, 151.0; Sedov 2 M 13.5, 13.3; clustered 2 M 19.1, 19.8; clustered 200 k 10.5,
-// 10.9; 32 k uniform 0.475, 0.50)
+// resident blocks per SM the search is compiled for: more warps where there are tiles of similar
+// cost for all of them many times over, else more registers for each, which shortens the tiles
+// that the others wait for (search_many has the line)
 constexpr int kSearchFew = 5, kSearchMany = 7;
 // the sums wait for scattered reads: a lane has both names of a step in flight, and five blocks
 // of four warps leave it the registers for that (Sedov 2 M, 19 M in 512 boxes, ms per call: one
@@ -1735,6 +1734,17 @@ static SumArgs sum_args(sph_ctx *ctx, sph_particles *parts)
 constexpr size_t kSearchSmem = (kListThreads / 32) * (16 * (size_t)kSearchF4 + 4 * 33);
 static_assert(kSearchSmem <= 48 * 1024, "no opt-in needed");
 
+// Uniform matter: ms per call with 5 blocks and with 7, 262,144 particles 3.55, 3.63; 524,288 5.64,
+// 5.64; 1 M 9.42, 9.33; 2 M 17.2, 16.9; the point explosion, 512,000 4.21, 4.24; 1 M 6.94, 6.91; 2 M
+// 13.3, 13.1.  Adaptive cells: one clustered box has a few tiles with the longest lists and takes
+// 5 at every size (500,000 8.8, 9.3; 2 M 17.0, 17.3; 4 M 31.0, 31.8; 8 M 58.5, 60.4); batches of
+// 37,000 a box, 16 boxes 9.4, 9.8; 64 22.4, 22.1; 160 52.4, 51.4; 512 152.8, 149.5.
+static bool search_many(const sph_ctx *ctx)
+{
+    if (ctx->adaptive) return ctx->n >= 2000000 && ctx->n_boxes >= 64;
+    return ctx->n >= 1000000;
+}
+
 // Pass `pass` (below kListPasses) of a density call: lists for the active targets; a pass
 // after the first runs only if the one before left targets.  pass < 0: the force pass's own
 // search, at the converged h, where the lists of the density passes do not serve.
@@ -1781,7 +1791,7 @@ int run_search(sph_ctx *ctx, sph_particles *parts, int pass, bool all)
     a.grow = force ? 1.f : ctx->lists.grow;
     a.wbits = name_bits(ctx);
     a.force = force ? 1 : 0;
-    const bool many = ctx->n >= (ctx->adaptive ? 8000000 : 1000000);
+    const bool many = search_many(ctx);
     const int g = list_grid(ctx, kListThreads, many ? kSearchMany : kSearchFew);
     cudaEvent_t end = nullptr;
     timer_begin(ctx, force ? 1 : 0, &end);
