@@ -1053,7 +1053,7 @@ static int do_steps(sph_ctx *ctx, sph_particles *parts, int n_steps, double dt, 
         if (rc) return rc;
     }
     sph_ctx::GraphKey key{*parts, dt > 0 ? dt : 0.0, ctx->n, ctx->grid.n_cells, ctx->grid.key_bits, passes, ctx->tile_w,
-                          tree_sig, ctx->sym_force, lists ? ctx->lists.pages : nullptr, lists ? ctx->lists.cap_pages : 0};
+                          tree_sig, ctx->sym_force, lists ? ctx->lists.made : 0};
     if (!ctx->step_exec || !(key == ctx->graph_key)) {
         if (!ctx->cap_stream) SPH_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
         const uint32_t flags = ctx->p.flags;

@@ -204,6 +204,7 @@ struct ListPool {
     int *rows = nullptr;        // 4 x cap: targets left by the last two passes, grown, dirty
     uint8_t *mark = nullptr;    // dirty targets of the present density call
     int64_t cap = 0, cap_pages = 0;
+    int64_t made = 0;           // allocations so far (names the present one)
     int64_t want = 0;           // pages that a captured step lacked
     // calls in a row whose lists did not fit the largest pool, the calls still to go by without a
     // search before one tries again, and the particle count of both
@@ -321,13 +322,12 @@ struct sph_ctx {
         int key_bits, passes, tile_w;
         uint64_t tree_sig;  // adaptive cells: arrays and capacities the captured build uses
         bool sym;           // symmetric force pass
-        const void *list_pages;  // neighbour-list pool (null: a step without lists)
-        int64_t list_cap;
+        int64_t lists;      // neighbour lists: the allocation they are in (0: a step without lists)
         bool operator==(const GraphKey &o) const
         {
             return memcmp(&parts, &o.parts, sizeof parts) == 0 && dt == o.dt && n == o.n && n_cells == o.n_cells &&
                    key_bits == o.key_bits && passes == o.passes && tile_w == o.tile_w && tree_sig == o.tree_sig &&
-                   sym == o.sym && list_pages == o.list_pages && list_cap == o.list_cap;
+                   sym == o.sym && lists == o.lists;
         }
     } graph_key{};
     int64_t graph_launches = 0;  // kernels in one captured step

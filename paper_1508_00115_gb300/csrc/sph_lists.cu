@@ -1582,7 +1582,9 @@ void free_lists(sph_ctx *ctx)
     cudaFree(P.radius);
     cudaFree(P.rows);
     cudaFree(P.mark);
+    const int64_t made = P.made;
     P = ListPool();
+    P.made = made;
 }
 
 // Arrays for the lists (never inside a capture): `pages` of them at least, five per particle to
@@ -1622,6 +1624,7 @@ bool ensure_lists(sph_ctx *ctx, int64_t pages)
         return room(&P.pages, sizeof(uint32_t) * kPage * (size_t)n) && room(&P.next, sizeof(int) * (size_t)n);
     };
     bool ok = true;
+    ++P.made;
     if (slots) {
         ok = room(&P.head, sizeof(int) * cap) && room(&P.cnt, sizeof(int) * cap) &&
              room(&P.radius, sizeof(float) * cap) && room(&P.rows, 4 * sizeof(int) * cap) &&

@@ -102,6 +102,13 @@ def test_leaf_too_large_for_its_names():
     s = oracle_state(g)
     check_density(g, s)
     check_force(g, s)
+    # captured steps: each search finds the leaf, the sums run without lists
+    ctx = binding.Context(2000, flags=binding.SPH_FLAG_ADAPTIVE | binding.SPH_FLAG_NGB_HASH, leaf_max=2)
+    parts = binding.Particles(d)
+    for _ in range(3):
+        ctx.steps(parts, 2, 1e-6)
+        assert ctx.stats()["graph_steps"] > 0
+        _check_call(ctx, parts)
 
 
 def _lowered(parts, share, factor, seed):
