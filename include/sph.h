@@ -91,8 +91,7 @@ typedef struct sph_ctx sph_ctx; /* opaque, library-owned */
                                 each with a list of the leaves within reach.  Top
                                 cells may number 1 or 2 per side (h < box/2).
                                 For h spanning decades (clustered matter).  Builds read
-                                tree sizes on the host, so sph_steps runs its steps
-                                one by one instead of replaying a CUDA graph. */
+                                tree sizes on the host, except inside sph_steps. */
 #define SPH_FLAG_TREE_H_GUESS 16u /* with SPH_FLAG_ADAPTIVE: the first cell build
                                 replaces every input h by an estimate from the number
                                 density n of the smallest tree node around it that

@@ -800,6 +800,21 @@ __global__ void k_leaf_active_tiles(const int2 *__restrict__ rng, const int *__r
     }
 }
 
+// Whether node N, moved by (dx, dy, dz), lies within reach of leaf A, whose own reach is hA.  A
+// list is counted and then written by two kernels, and by a warp or a thread, which all have
+// to decide alike: every rounding is spelled out, so that no kernel's compilation contracts
+// other products than another's.  (Where one more entry was written than counted, the next
+// leaf lost its first.)
+__device__ __forceinline__ bool within_reach(const TreeNode &A, const TreeNode &N, float dx, float dy, float dz, float hA,
+                                             float slack)
+{
+    const float gx = fmaxf(fmaxf(__fsub_rn(__fadd_rn(N.bx0, dx), A.bx1), __fsub_rn(A.bx0, __fadd_rn(N.bx1, dx))), 0.f);
+    const float gy = fmaxf(fmaxf(__fsub_rn(__fadd_rn(N.by0, dy), A.by1), __fsub_rn(A.by0, __fadd_rn(N.by1, dy))), 0.f);
+    const float gz = fmaxf(fmaxf(__fsub_rn(__fadd_rn(N.bz0, dz), A.bz1), __fsub_rn(A.bz0, __fadd_rn(N.bz1, dz))), 0.f);
+    const float reach = __fmaf_rn(fmaxf(hA, __fmul_rn(N.hmax, kTreeReach)), 1.f + 1e-5f, slack);
+    return __fmaf_rn(gx, gx, __fmaf_rn(gy, gy, __fmul_rn(gz, gz))) < __fmul_rn(reach, reach);
+}
+
 // Neighbour leaves of leaf `l`: walk the subtrees of the 27 top cells around its own,
 // keeping nodes whose bounding box is within reach.  COUNT: only count; else write
 // {offset between the leaf centres (FP32), neighbour leaf} from out[0].
@@ -814,10 +829,10 @@ __device__ int leaf_pairs(int l, const int *__restrict__ leaf_node, const TreeNo
     const BoxDev g = bxs[nb == 1 ? 0 : tbox_of_cell(A.top, bxs, nb)];
     const int nc = g.nc, loc = A.top - g.cell_off;
     const int ix = loc % nc, iy = (loc / nc) % nc, iz = loc / (nc * nc);
-    const float hA = A.hmax * kTreeReach;
+    const float hA = __fmul_rn(A.hmax, kTreeReach);
     // FP32 rounding of the boxes and offsets (a few ulps of the top cell) is covered
     // by a slack added to every reach
-    const float slack = 4.8e-7f * g.L32;
+    const float slack = __fmul_rn(4.8e-7f, g.L32);
     const double cAx = leaf_cen[3 * l], cAy = leaf_cen[3 * l + 1], cAz = leaf_cen[3 * l + 2];
     const double sideA = ldexp(g.L64, -A.level);
     double scale = sideA;
@@ -835,17 +850,13 @@ __device__ int leaf_pairs(int l, const int *__restrict__ leaf_node, const TreeNo
         const int root = top_node[g.cell_off + (jz * nc + jy) * nc + jx];
         if (root < 0) continue;
         // offset of the neighbour top cell's centre relative to A's (FP32, multiples of L)
-        const float dx = (float)ox * g.L32, dy = (float)oy * g.L32, dz = (float)oz * g.L32;
+        const float dx = __fmul_rn((float)ox, g.L32), dy = __fmul_rn((float)oy, g.L32), dz = __fmul_rn((float)oz, g.L32);
         int sp = 0;
         stack[sp++] = root;
         while (sp > 0) {
             const int id = stack[--sp];
             const TreeNode N = nodes[id];
-            const float gx = fmaxf(fmaxf(N.bx0 + dx - A.bx1, A.bx0 - (N.bx1 + dx)), 0.f);
-            const float gy = fmaxf(fmaxf(N.by0 + dy - A.by1, A.by0 - (N.by1 + dy)), 0.f);
-            const float gz = fmaxf(fmaxf(N.bz0 + dz - A.bz1, A.bz0 - (N.bz1 + dz)), 0.f);
-            const float reach = fmaxf(hA, N.hmax * kTreeReach) * (1.f + 1e-5f) + slack;
-            if (gx * gx + gy * gy + gz * gz >= reach * reach) continue;
+            if (!within_reach(A, N, dx, dy, dz, hA, slack)) continue;
             if (N.child < 0) {
                 if (!COUNT) {
                     const int b = node_leaf[id];
@@ -941,8 +952,8 @@ __device__ void walk_leaf(const WalkArgs &a, int l, int2 *st)
     const BoxDev g = a.bxs[a.nb == 1 ? 0 : tbox_of_cell(A.top, a.bxs, a.nb)];
     const int nc = g.nc, loc = A.top - g.cell_off;
     const int ix = loc % nc, iy = (loc / nc) % nc, iz = loc / (nc * nc);
-    const float hA = A.hmax * kTreeReach;
-    const float slack = 4.8e-7f * g.L32;
+    const float hA = __fmul_rn(A.hmax, kTreeReach);
+    const float slack = __fmul_rn(4.8e-7f, g.L32);
     const float sideA = ldexpf(g.L32, -A.level);
     // roots: the non-empty top cells around A's, item = {root node, image index}
     int sp;
@@ -982,12 +993,8 @@ __device__ void walk_leaf(const WalkArgs &a, int l, int2 *st)
         const int ox = o % 3 - 1, oy = (o / 3) % 3 - 1, oz = o / 9 - 1;
         if (it.x >= 0) {
             const TreeNode N = a.nodes[it.x];
-            const float dx = (float)ox * g.L32, dy = (float)oy * g.L32, dz = (float)oz * g.L32;
-            const float gx = fmaxf(fmaxf(N.bx0 + dx - A.bx1, A.bx0 - (N.bx1 + dx)), 0.f);
-            const float gy = fmaxf(fmaxf(N.by0 + dy - A.by1, A.by0 - (N.by1 + dy)), 0.f);
-            const float gz = fmaxf(fmaxf(N.bz0 + dz - A.bz1, A.bz0 - (N.bz1 + dz)), 0.f);
-            const float reach = fmaxf(hA, N.hmax * kTreeReach) * (1.f + 1e-5f) + slack;
-            if (gx * gx + gy * gy + gz * gz < reach * reach) {
+            const float dx = __fmul_rn((float)ox, g.L32), dy = __fmul_rn((float)oy, g.L32), dz = __fmul_rn((float)oz, g.L32);
+            if (within_reach(A, N, dx, dy, dz, hA, slack)) {
                 if (N.child < 0) {
                     emit = true;
                     level = N.level;

@@ -498,3 +498,30 @@ def test_adaptive_steps_deterministic(graph):
         out.append(g)
     for k in ("x", "vx", "u", "rho", "h", "ax", "ay", "az", "dudt", "vsig", "n_ngb", "perm", "ngb_hash"):
         assert np.array_equal(out[0][k], out[1][k]), k
+
+
+@pytest.mark.parametrize("leaf", [1, 8])
+def test_leaf_lists_where_distances_tie_with_the_reach(leaf):
+    """A lattice whose h puts the leaves' reach within a few roundings of a lattice distance, so
+    that thousands of pairs of leaves are decided by the last bit: the lists are counted, then
+    written, and every particle's neighbours have to be the lattice vectors within h."""
+    from paper_1508_00115_gb300 import binding
+    side = 16
+    d = inputs.lattice(side, 1.0, jitter=0.0, seed=1)
+    n = side ** 3
+    k = np.arange(side)
+    k = np.minimum(k, side - k)
+    v2 = (k[:, None, None] ** 2 + k[None, :, None] ** 2 + k[None, None, :] ** 2) / side ** 2
+    ctx = binding.Context(n, flags=binding.SPH_FLAG_ADAPTIVE, leaf_max=leaf, cell_factor=1.25, max_h_iter=1)
+    parts = binding.Particles(d)
+    for v in ((2, 1, 1), (3, 0, 0), (2, 2, 1), (3, 2, 1)):
+        r = np.sqrt(sum(c * c for c in v)) / side
+        for below in (0.0, 2.4e-7, 4.8e-7):  # (the boxes' pads of 1.2e-7 of a top cell, once per axis)
+            h0 = np.float32((r - below * 0.25) / (1.15 * (1 + 1e-5)))
+            for step in range(-6, 7):
+                h = h0 + np.float32(step) * np.spacing(h0)
+                parts.t["h"].fill_(float(h))
+                ctx.build_cells(parts)
+                ctx.density(parts, allow_not_converged=True)
+                assert (parts.t["n_ngb"].cpu().numpy() == int((v2 < float(h) ** 2).sum()) - 1).all(), (v, below, step)
+                assert float(parts.t["h"].min()) == float(h)
