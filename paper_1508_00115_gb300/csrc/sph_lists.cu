@@ -15,8 +15,8 @@
 // grid, the slot and the stencil cell it was met in, with adaptive cells the entry of the
 // target's leaf list and the index in that leaf.  Pages come from one pool, handed out by
 // an atomic counter; a list's content and order depend on the cells only, so every sum is the
-// same on every run.  When the pool runs out, the flag STALE_OVERFLOW tells
-// the kernels of sph_pairs.cu to run instead.
+// same on every run.  When the pool runs out, C_STALE tells the kernels of
+// sph_pairs.cu to run instead.
 #include <cuda_fp16.h>
 
 #include <algorithm>

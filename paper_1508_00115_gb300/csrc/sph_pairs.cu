@@ -6,7 +6,8 @@
 // Here without neighbour lists: every pass searches for itself.  sph_lists.cu runs both over
 // lists instead, wherever its lists apply; these kernels run where they do not (the axis
 // sweep, uniform grids beyond 2^25 slots, adaptive cells before a density call has
-// converged, lists that found no room), and the symmetric force pass always.
+// converged, a guess of h whose lists would be far too long, lists that found no room),
+// and the symmetric force pass always.
 //
 // Work decomposition (replaces the paper's self/pair tasks and task scheduler):
 // a tile is up to TW (16 or 32) target particles of one cell, one lane per
