@@ -1178,11 +1178,7 @@ __global__ void __launch_bounds__(kSumThreads, kSumBlocks) k_density_l(DensityLi
                 float hn = hi;
                 unsigned flag = 0u;
                 if (!conv) {
-                    // Newton step, at most a factor 2 either way; a step that leaves a
-                    // two-sided bracket is replaced by its geometric middle
-                    hn = dnw_dh > 0.f ? hi - g / dnw_dh : (g < 0.f ? 2.f * hi : 0.5f * hi);
-                    hn = fminf(fmaxf(hn, 0.5f * hi), 2.f * hi);
-                    if (lo > 0.f && up < kHUnbounded && !(hn > lo && hn < up)) hn = sqrtf(lo) * sqrtf(up);
+                    hn = next_h(hi, g, dnw_dh, lo, up);
                     if (LIST) {
                         // adaptive cells: h up to just below half the box; beyond what its
                         // leaf's list or the adjacent top cells hold the cells are built

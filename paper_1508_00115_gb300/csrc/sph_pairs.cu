@@ -646,11 +646,7 @@ __global__ void __launch_bounds__(kPairThreads, kDensityBlocks) k_density(Densit
                 conv = lo > 0.f && up < kHUnbounded && up - lo <= kHResolution * lo;
             }
             if (!conv && !a.last_pass) {
-                // Newton step, at most a factor 2 either way; a step that leaves a
-                // two-sided bracket is replaced by its geometric middle
-                float hn = dnw_dh > 0.f ? hi - g / dnw_dh : (g < 0.f ? 2.f * hi : 0.5f * hi);
-                hn = fminf(fmaxf(hn, 0.5f * hi), 2.f * hi);
-                if (lo > 0.f && up < kHUnbounded && !(hn > lo && hn < up)) hn = sqrtf(lo) * sqrtf(up);
+                float hn = next_h(hi, g, dnw_dh, lo, up);
                 flag = 1u;
                 if (LIST) {
                     // adaptive cells: h up to just below half the box (the minimum

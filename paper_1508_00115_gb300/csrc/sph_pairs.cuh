@@ -17,6 +17,8 @@ constexpr float kHUnbounded = 3e38f;
 // of h, so that for particles whose N_w is very sensitive to h a tolerance far below
 // 1e-5 may have no FP32 h that meets it
 constexpr float kHResolution = 4.76837158e-7f;
+// a little less: the nudge of an h whose Newton step is below its last bit
+constexpr float kHNudge = 4.3e-7f;
 
 // Neighbour cells in visiting order: the own cell, then each of the 13 directions
 // of a half stencil followed by its opposite, so that every staged batch mixes
@@ -167,6 +169,20 @@ __device__ __forceinline__ unsigned long long warp_sum_ull(unsigned long long v)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     return v;
+}
+
+// The next iterate of N_w(h) = N_ngb from h, where N_w misses it by g and lo, up bracket the
+// root: Newton's step, at most a factor 2 either way; a step that leaves a two-sided bracket is
+// replaced by its geometric middle.  Where N_w is so steep that the step rounds to
+// nothing (a kernel whose edge is in a halo: two neighbouring floats miss h_tol on either side
+// of the root), h goes past the root, so that the bracket closes; it would stay for ever.
+__device__ __forceinline__ float next_h(float h, float g, float dnw_dh, float lo, float up)
+{
+    float hn = dnw_dh > 0.f ? h - g / dnw_dh : (g < 0.f ? 2.f * h : 0.5f * h);
+    hn = fminf(fmaxf(hn, 0.5f * h), 2.f * h);
+    if (hn == h) hn = g < 0.f ? h * (1.f + kHNudge) : h * (1.f - kHNudge);
+    if (lo > 0.f && up < kHUnbounded && !(hn > lo && hn < up)) hn = sqrtf(lo) * sqrtf(up);
+    return hn;
 }
 
 __device__ __forceinline__ int wrapc(int j, int nc) { return j < 0 ? j + nc : (j >= nc ? j - nc : j); }

@@ -525,3 +525,40 @@ def test_leaf_lists_where_distances_tie_with_the_reach(leaf):
                 ctx.density(parts, allow_not_converged=True)
                 assert (parts.t["n_ngb"].cpu().numpy() == int((v2 < float(h) ** 2).sum()) - 1).all(), (v, below, step)
                 assert float(parts.t["h"].min()) == float(h)
+
+
+@pytest.mark.parametrize("second", [False, True])
+def test_roots_between_two_floats(second):
+    """Sparse particles whose kernels end in a dense clump: N_w moves by more than h_tol from one
+    FP32 h to the next, and a Newton step from one side of the root may round to nothing.  Every h
+    has its root within the resolution of the iteration (2^-21), with lists (second call) and
+    without."""
+    from paper_1508_00115_gb300 import binding
+    rng = np.random.default_rng(131)
+    n, clump = 4400, 4000
+    d = inputs.uniform(n, seed=132)
+    for k in ("x", "y", "z"):
+        d[k][:clump] = 0.5 + 1e-3 * (rng.random(clump) - 0.5)
+        d[k][clump:] = 0.5 + 0.3 * (rng.random(n - clump) - 0.5)
+    tol = 2e-7
+    ctx = binding.Context(n, flags=_flags() | binding.SPH_FLAG_TREE_H_GUESS, h_tol=tol, max_h_iter=60)
+    parts = binding.Particles(d)
+    for _ in range(2 if second else 1):
+        ctx.build_cells(parts)
+        ctx.density(parts)
+        if second:
+            parts.t["h"] *= 1.01
+    if second:
+        ctx.build_cells(parts)
+        ctx.density(parts)
+    g = parts.numpy()
+    g["perm"] = ctx.permutation()
+    t = np.flatnonzero(g["perm"] >= clump)
+    nw = []
+    for f in (1.0, 1.0 - 2.0 ** -21, 1.0 + 2.0 ** -21):
+        s = oracle_state(dict(g, h=g["h"].astype(np.float64) * f))
+        nw.append(oracle.density_at_h(s, targets=t)["nw"] / 48.0 - 1.0)
+    eps = 4e-7  # rounding of the FP32 sums
+    met = np.abs(nw[0]) <= tol + eps
+    assert (met | ((nw[1] <= eps) & (nw[2] >= -eps))).all()
+    assert (~met).any()  # (such roots are there)
