@@ -533,7 +533,7 @@ static int do_density(sph_ctx *ctx, sph_particles *parts, int32_t *iters_out)
                 ++rebinned;
                 before = iters;
                 since = 0;
-                use_lists = turn && settled;
+                use_lists = turn && settled && lists_apply(ctx);  // (a growth may have lost the pool)
                 fresh = true;
                 again = some_done = partial = false;
                 rc = density_begin(ctx, ctx->bin_mode, turn);  // slots were permuted
